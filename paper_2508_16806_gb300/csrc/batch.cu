@@ -374,7 +374,7 @@ __global__ void kb_step_ctrl(Ctrl* ctrl, int B, const int32_t* t0K, const int32_
         dx2 = warp_range_sum(partT, t0T[k], t0T[k + 1]);
         inter = warp_range_sum(partT + ntT, t0T[k], t0T[k + 1]);
     }
-    if ((threadIdx.x & 31) == 0) step_decide(c, c->adaptive, dy2, dx2, inter);
+    if ((threadIdx.x & 31) == 0) step_decide(c, c->adaptive, dy2, dx2, inter, nullptr, global_ns());
 }
 
 // ---------------------------------------------------------------- check kernels
@@ -492,7 +492,10 @@ __global__ void kb_check_ctrl(Ctrl* ctrl, int B, const int32_t* t0K, const int32
     for (int q = 0; q < kColQ; ++q)
         cc[q] = q < kColSums ? warp_range_sum(partC + (size_t)q * ntT, t0T[k], t0T[k + 1])
                              : warp_range_max(partC + (size_t)q * ntT, t0T[k], t0T[k + 1]);
-    if ((threadIdx.x & 31) == 0) check_decide(c, r, cc, nullptr);
+    // lane 0 holds the totals
+    for (int q = 0; q < kRowQ; ++q) r[q] = __shfl_sync(0xffffffffu, r[q], 0);
+    for (int q = 0; q < kColQ; ++q) cc[q] = __shfl_sync(0xffffffffu, cc[q], 0);
+    check_decide(c, r, cc, nullptr);
 }
 
 template <typename T>
@@ -593,6 +596,8 @@ __global__ void kb_init_ctrl(Ctrl* ctrl, int B, const double* normK, const doubl
                 c.cand_avg = 0;
             }
         }
+        c.next_check = (c.k / c.check_every + 1) * c.check_every;
+        c.romega = 1.0 / c.omega;
         refresh_scalars(c);
         ctrl[k] = c;
     }
@@ -1139,7 +1144,7 @@ lp_status batch_solve_t(BatchHandle* bh, const lp_opts* o, lp_result* rs,
     tmpl.beta_n = o->beta_necessary;
     tmpl.beta_a = o->beta_artificial;
     tmpl.eps_zero = o->eps_zero;
-    tmpl.time_limit_ns = o->time_limit_s * 1e9;
+    tmpl.time_limit_ns = limit_ns(o->time_limit_s);
     tmpl.max_iters = o->max_iters;
     tmpl.status = kRunning;
     tmpl.first = 1;

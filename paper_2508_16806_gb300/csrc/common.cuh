@@ -18,6 +18,8 @@ constexpr int kNT = 256;          // threads of an SpMV row-block
 constexpr int kEW = 256;          // threads of an elementwise block
 constexpr int kEWGrid = 1216;     // elementwise grid cap: 152 SMs x 8 resident blocks
 constexpr int kCtlNT = 512;       // threads of a control (single-block) kernel
+constexpr int kCheckNT = 512;     // threads and largest grid of the KKT-check reductions: two
+constexpr int kCheckGrid = 304;   // blocks per SM (more blocks only add partial sums)
 // KKT-check reductions: row side 11 sums + 2 maxima, column side 15 sums + 1 maximum
 constexpr int kRowSums = 11, kRowMax = 2, kRowQ = kRowSums + kRowMax;
 constexpr int kColSums = 15, kColMax = 1, kColQ = kColSums + kColMax;
@@ -43,6 +45,7 @@ struct Ctrl {
     double pend_w;       // eta of the last accepted iterate not yet added to the averages
     double W;            // sum of eta over the iterates in the averages
     double Winv;         // 1 / W (0 while W = 0)
+    double romega;       // 1 / omega
     // restart state (Section 2.4.2)
     double kkt_anchor, kkt_prev;
     // last check
@@ -50,7 +53,7 @@ struct Ctrl {
     // options
     double tol, beta_s, beta_n, beta_a, eps_zero;
     double qnorm, cnorm;         // ||q||_2, ||c||_2 of the unscaled problem
-    double time_limit_ns;
+    long long time_limit_ns;
     double infeas_tol;   // Algorithm 6 tolerance (normalised directions)
     // restarted Halpern variant: reflection rho, the fixed-point residual
     // ||z - T(z)||_P of the last iteration, of the first iteration of the epoch,
@@ -58,6 +61,7 @@ struct Ctrl {
     double reflect, fpr, fpr0, fpr_prev;
     // counters
     long long k, attempts, epoch_k, restarts, max_iters, t0_ns, trace_len, trace_cap;
+    long long next_check;   // the next multiple of check_every (a 64-bit remainder per attempt is slow)
     int cur;             // which half of each double buffer holds the current iterate
     int skip;            // step kernels return at once (check pending or done)
     int want_check;      // the check kernels run
@@ -99,9 +103,24 @@ struct Ctrl {
     StepScalars<double> s64;
 };
 
+// A time limit in seconds as nanoseconds (saturating).
+inline long long limit_ns(double s)
+{
+    return s >= 9.0e9 ? (long long)9e18 : (long long)(s * 1e9);
+}
+
+// n / d for rd = 1 / d (correctly rounded): the product with rd corrected by its
+// residual, which rounds correctly (Markstein, 1990).  Three fused multiply-adds
+// (200 cycles of GB300's FP64 unit) instead of a division (1,500).
+__host__ __device__ inline double div_by(double n, double d, double rd)
+{
+    const double q = n * rd;
+    return fma(fma(-d, q, n), rd, q);
+}
+
 __host__ __device__ inline void refresh_scalars(Ctrl& c)
 {
-    const double tau = c.eta / c.omega, sigma = c.eta * c.omega;
+    const double tau = div_by(c.eta, c.omega, c.romega), sigma = c.eta * c.omega;
     const double lam = (double)(c.epoch_k + 1) / (double)(c.epoch_k + 2);
     const double ha = lam * (1.0 + c.reflect), hb = lam * c.reflect, hg = 1.0 - lam;
     c.s64 = StepScalars<double>{tau, sigma, c.pend_w, c.Winv, ha, hb, hg};
@@ -162,6 +181,32 @@ struct SplitRows {
     const int32_t* wend = nullptr;
 };
 
+// Resident iterations (resident.cuh): row classes of one orientation and the
+// plan of one precision.
+struct ResSide {
+    int chunk = 0;                    // cluster form: entries of the vector that a block owns
+    int lgmin = 0;                    // log2 of the fewest lanes per row
+    const int32_t* cptr = nullptr;    // [blocks + 1] first slice of each block
+    const int32_t* eptr = nullptr;    // [blocks + 1] first entry
+    const int32_t* rptr = nullptr;    // [blocks + 1] first slot (a row's place in its block)
+    const int4* slice = nullptr;      // first entry in its block, steps, log2 of the lanes per
+                                      // row, first slot in its block
+    const int32_t* row = nullptr;     // the row of each slot (-1: none)
+    const int32_t* sidx = nullptr;    // column indices of the entries (32 per step)
+    int nslice = 0;
+    int max_entry = 0, max_slice = 0, max_slot = 0;   // of any block
+};
+struct ResPlan {
+    bool on = false;
+    bool cluster = false;             // one cluster with x and y in shared memory
+    int ncta = 0, threads = 0;
+    size_t smem = 0;
+    ResSide K, T;
+    void *svalK = nullptr, *svalT = nullptr;   // values of the slices' entries
+    void* slots = nullptr;            // grid form: barrier arrivals [2][ncta]
+    unsigned int* seq = nullptr;      // barriers met by earlier launches, arrivals counted
+};
+
 // State and scaled data of one precision T (double or float).
 template <typename T>
 struct Engine {
@@ -192,6 +237,7 @@ struct Engine {
     int npK = 0, npT = 0;                       // partials of the two launches: grid + split rows
     SchedParams schedK, schedT;                 // parameters of the two schedules
     bool tuned = false;                         // schedules chosen by the autotuner
+    ResPlan res;                                // resident iterations (small LPs)
     // Ruiz factors R, C and their reciprocals in this precision (KKT checks)
     T* Rt = nullptr; T* Ct = nullptr; T* Rinv = nullptr; T* Cinv = nullptr;
     // reduction partials
@@ -325,6 +371,70 @@ __device__ __forceinline__ void block_partials(const double (&v)[NQ], double* pa
             t = warp_sum(t);
             if (lane == 0) part[(size_t)q * stride + blockIdx.x] = t;
         }
+    }
+}
+
+// Sums of 16 values per lane over the warp: lane l returns the total of value
+// l % 16 (fixed order).  Each round halves the values a lane carries: 16 FP64
+// additions instead of the 80 of 16 separate trees (an addition takes the FP64
+// unit of a quarter SM for 64 cycles).
+__device__ __forceinline__ double warp_sums16(double (&v)[16])
+{
+    const int lane = threadIdx.x & 31;
+#pragma unroll
+    for (int k = 8; k >= 1; k >>= 1) {
+        const bool up = lane & k;
+#pragma unroll
+        for (int i = 0; i < k; ++i) {
+            const double send = up ? v[i] : v[i + k], keep = up ? v[i + k] : v[i];
+            v[i] = keep + __shfl_xor_sync(0xffffffffu, send, k);
+        }
+    }
+    return v[0] + __shfl_xor_sync(0xffffffffu, v[0], 16);
+}
+
+// Maximum of non-negative values over the warp (as integers, which order like
+// them; a NaN counts as the largest).
+__device__ __forceinline__ double warp_max_nonneg(double v)
+{
+    unsigned long long b = (unsigned long long)__double_as_longlong(v);
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+        const unsigned long long u = __shfl_xor_sync(0xffffffffu, b, o);
+        b = u > b ? u : b;
+    }
+    return __longlong_as_double((long long)b);
+}
+
+// Block sums of NS <= 16 and maxima of NM non-negative values per thread:
+// part[q * stride + blockIdx.x], the sums first.
+template <int NS, int NM, int NT, typename T>
+__device__ __forceinline__ void block_check_partials(const T (&v)[NS], const T (&mx)[NM],
+                                                     double* part, int stride)
+{
+    __shared__ double ss[NT / 32][16];
+    __shared__ double sm[NT / 32][NM];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    double d[16];
+#pragma unroll
+    for (int q = 0; q < 16; ++q) d[q] = q < NS ? (double)v[q] : 0.0;
+    const double s = warp_sums16(d);
+    if (lane < 16) ss[warp][lane] = s;
+#pragma unroll
+    for (int q = 0; q < NM; ++q) {
+        const double t = warp_max_nonneg((double)mx[q]);
+        if (lane == 0) sm[warp][q] = t;
+    }
+    __syncthreads();
+    if (threadIdx.x < NS) {
+        double t = 0.0;
+        for (int w = 0; w < NT / 32; ++w) t += ss[w][threadIdx.x];
+        part[(size_t)threadIdx.x * stride + blockIdx.x] = t;
+    } else if (threadIdx.x >= 32 && threadIdx.x < 32 + NM) {
+        const int q = threadIdx.x - 32;
+        double t = 0.0;
+        for (int w = 0; w < NT / 32; ++w) t = fmax(t, sm[w][q]);
+        part[(size_t)(NS + q) * stride + blockIdx.x] = t;
     }
 }
 
@@ -466,6 +576,12 @@ lp_status extract_solution_ex(Handle* h, double* x, double* y, int space, double
 lp_status sum_of_squares(Handle* h, const double* v, int64_t count, double* out_host);
 template <typename T>
 lp_status profile_step(Handle* h, int reps, double* ms, double* bytes);
+// resident.cu: the plan of an engine (res.on false: the LP is too large), the
+// attempts of one check period, Algorithm 2 from ones (||K b / ||b|| ||^2 -> out)
+template <typename T> lp_status res_plan(Handle* h);
+template <typename T> lp_status res_values(Handle* h);   // the slices' values from val, tval
+template <typename T> lp_status launch_res_period(Handle* h, cudaStream_t st, bool halpern);
+lp_status launch_res_power(Handle* h, cudaStream_t st, int iters, double* out);
 // grad.cu
 lp_status run_grad(Handle* h, const lp_opts* o, int K_iters, int ckpt, const double* gxK,
                    double* dc, double* dq, double* dvals, double* xK, int space,

@@ -115,6 +115,30 @@ struct ColCheck {
     }
 };
 
+// The bit pattern of a value as an integer that orders like it (a sign bit turns
+// the order of the rest round; NaNs lie beyond the infinities).
+__device__ __forceinline__ long long order_key(double a)
+{
+    const long long b = __double_as_longlong(a);
+    return b ^ (long long)((unsigned long long)(b >> 63) >> 1);
+}
+
+// n / d where both are of ordinary size (and n may be 0): an FP32 reciprocal
+// refined by two Newton steps, the quotient corrected by its residual (Markstein,
+// 1990).  About 600 cycles of the deciding thread, on every attempt's critical
+// path, instead of the 1,500 of a division.
+__device__ __forceinline__ double quotient(double n, double d)
+{
+    const int en = (int)((unsigned long long)__double_as_longlong(n) >> 52) & 2047;
+    const int ed = (int)((unsigned long long)__double_as_longlong(d) >> 52) & 2047;
+    if (ed < 923 || ed > 1123 || (n != 0.0 && (en < 523 || en > 1523))) return n / d;
+    double r = (double)__frcp_rn((float)d);
+    r = fma(r, fma(-d, r, 1.0), r);
+    r = fma(r, fma(-d, r, 1.0), r);
+    const double q = n * r;
+    return fma(fma(-d, q, n), r, q);
+}
+
 // Whether the check kernels evaluate Algorithm 6 for this control block.
 __device__ __forceinline__ bool infeas_active(const Ctrl& c)
 {
@@ -124,15 +148,19 @@ __device__ __forceinline__ bool infeas_active(const Ctrl& c)
 // Algorithm 5 decision (or the plain swap of a fixed step), by one thread.
 // The paper's k is read as the 1-based index of the iteration being taken.
 // Halpern iterations (fixed step) also record the fixed-point residual.
+// now: the device clock (every block of a launch that decides redundantly takes
+// the same reading).  lazy: 1 / W and the step scalars are left to the caller.
 __device__ __forceinline__ void step_decide(Ctrl* ctrl, int adapt, double dy2, double dx2, double inter,
-                                            double* eta_bar_out = nullptr)
+                                            double* eta_bar_out, unsigned long long now,
+                                            bool lazy = false)
 {
     const double eta = ctrl->eta, omega = ctrl->omega;
     bool accept = true;
     double eta_next = eta;
     if (adapt) {
-        const double movement = omega * dx2 + dy2 / omega;
-        const double eta_bar = inter != 0.0 ? movement / (2.0 * fabs(inter)) : INFINITY;
+        const double movement = omega * dx2 + div_by(dy2, omega, ctrl->romega);
+        const double eta_bar =
+            order_key(fabs(inter)) != 0 ? quotient(movement, 2.0 * fabs(inter)) : INFINITY;
         if (eta_bar_out) *eta_bar_out = eta_bar;
         // (k + 1) of the paper with its k 1-based: accepted iterations + 2; the two
         // factors come from the period's table when the check filled one
@@ -148,9 +176,12 @@ __device__ __forceinline__ void step_decide(Ctrl* ctrl, int adapt, double dy2, d
         }
         const double e1 = f3 * eta_bar;
         const double e2 = f6 * eta;
-        eta_next = e1 < e2 ? e1 : e2;
-        accept = eta <= eta_bar;
-        if (!isfinite(movement) || isnan(inter)) {
+        // comparisons of values that are not negative, on their bit patterns: an FP64
+        // comparison takes the FP64 unit for about 100 cycles (NaN: rejected below)
+        eta_next = order_key(e1) < order_key(e2) ? e1 : e2;
+        accept = order_key(eta) <= order_key(eta_bar);
+        if (order_key(fabs(movement)) >= 0x7ff0000000000000ll ||
+            order_key(fabs(inter)) > 0x7ff0000000000000ll) {
             ctrl->status = LP_NUMERICAL_ERROR;
             ctrl->done = 1;
             ctrl->skip = 1;
@@ -160,7 +191,7 @@ __device__ __forceinline__ void step_decide(Ctrl* ctrl, int adapt, double dy2, d
     if (ctrl->halpern) {
         // fixed-point residual of this iteration in the PDHG metric:
         // ||(dx, dy)||_P^2 = ||dx||^2 / tau + ||dy||^2 / sigma + 2 dy^T K dx
-        const double r2 = (omega * dx2 + dy2 / omega) / eta + 2.0 * inter;
+        const double r2 = quotient(omega * dx2 + div_by(dy2, omega, ctrl->romega), eta) + 2.0 * inter;
         if (!isfinite(r2)) {
             ctrl->status = LP_NUMERICAL_ERROR;
             ctrl->done = 1;
@@ -177,29 +208,31 @@ __device__ __forceinline__ void step_decide(Ctrl* ctrl, int adapt, double dy2, d
         ctrl->epoch_k += 1;
         ctrl->pend_w = ctrl->halpern ? 0.0 : eta;
         ctrl->W += eta;
-        ctrl->Winv = 1.0 / ctrl->W;
+        if (!lazy) ctrl->Winv = 1.0 / ctrl->W;
         ctrl->rejects = 0;
     } else {
         ctrl->pend_w = 0.0;
         ctrl->rejects += 1;
     }
     ctrl->eta = eta_next;
-    refresh_scalars(*ctrl);
+    if (!lazy) refresh_scalars(*ctrl);
     // a check follows an accepted iteration that completes a check period (or
     // reaches max_iters); a rejected attempt never checks (the iterate did not move)
-    if (accept && (ctrl->k % ctrl->check_every == 0 || ctrl->k >= ctrl->max_iters)) {
+    if (accept && (ctrl->k >= ctrl->next_check || ctrl->k >= ctrl->max_iters)) {
+        if (ctrl->k >= ctrl->next_check) ctrl->next_check += ctrl->check_every;
         ctrl->want_check = 1;
         ctrl->skip = 1;
     }
     // guards that end the device loop even if no check is reached: Algorithm 5
     // accepts once eta <= 1/||K||, so a long run of rejections means broken
     // arithmetic; the wall-clock limit is also enforced per attempt.
-    if (ctrl->rejects > 1000 || !(eta_next > 0.0)) {
+    if (ctrl->rejects > 1000 || order_key(eta_next) <= 0 ||
+        order_key(eta_next) > 0x7ff0000000000000ll) {
         ctrl->status = LP_NUMERICAL_ERROR;
         ctrl->done = 1;
         ctrl->skip = 1;
         ctrl->want_check = 0;
-    } else if ((double)(global_ns() - (unsigned long long)ctrl->t0_ns) > ctrl->time_limit_ns) {
+    } else if ((long long)now - ctrl->t0_ns > ctrl->time_limit_ns) {
         ctrl->status = LP_TIME_LIMIT;
         ctrl->done = 1;
         ctrl->skip = 1;
@@ -207,52 +240,98 @@ __device__ __forceinline__ void step_decide(Ctrl* ctrl, int adapt, double dy2, d
     }
 }
 
+// One record of the attempt log (kAttemptFields), after the decision.
+__device__ __forceinline__ void log_attempt(Ctrl* ctrl, long long k0, double eta, double eta_bar,
+                                            double omega, bool sums, double dx2, double dy2,
+                                            double inter, bool write = true)
+{
+    if (write && ctrl->alog && ctrl->alog_len < ctrl->alog_cap) {
+        double* r = ctrl->alog + kAttemptFields * ctrl->alog_len;
+        r[0] = (double)k0; r[1] = eta; r[2] = eta_bar; r[3] = ctrl->eta;
+        r[4] = ctrl->k != k0 ? 1.0 : 0.0; r[5] = omega;
+        r[6] = sums ? dx2 : NAN; r[7] = sums ? dy2 : NAN; r[8] = sums ? inter : NAN;
+    }
+    ctrl->alog_len += 1;
+}
+
 // KKT_omega (Section 2.4.2) of the current point and of the average, the
 // restart candidate, the termination test on the unscaled problem (Section
 // 2.3.2), the three restart criteria (Section 2.4.2) and Algorithm 4, by one
-// thread.  r[kRowQ] and cc[kColQ] are the row- and column-side reductions of
-// k_check_rows / k_check_cols.
+// warp (all lanes call it; lane 0 updates the control block).  r[kRowQ] and
+// cc[kColQ] are the row- and column-side reductions of k_check_rows /
+// k_check_cols.  The square roots are taken by the lanes side by side, then the
+// divisions: one after another in one thread they took 12 us of every check.
 __device__ __forceinline__ void check_decide(Ctrl* ctrl, const double* r, const double* cc,
                                              lp_trace_rec* trace)
 {
+    const int lane = threadIdx.x & 31;
     const double w = ctrl->omega;
     // current
     const double pobj_c = cc[2], dobj_c = r[2] + cc[3];
     const double gap_c = dobj_c - pobj_c;
-    const double kkt_c = sqrt(w * w * r[0] + cc[0] / (w * w) + gap_c * gap_c);
     // average
     const double pobj_a = cc[7], dobj_a = r[6] + cc[8];
     const double gap_a = dobj_a - pobj_a;
+    double arg = 0.0;
+    if (lane < 2) {
+        const double rr = lane ? r[4] : r[0], dd = lane ? cc[5] : cc[0], g = lane ? gap_a : gap_c;
+        arg = w * w * rr + dd / (w * w) + g * g;
+    }
+    if (lane == 2) arg = r[1];
+    if (lane == 3) arg = r[5];
+    if (lane == 4) arg = cc[1];
+    if (lane == 5) arg = cc[6];
+    if (lane == 6) arg = cc[10];
+    if (lane == 7) arg = r[9] + cc[13];
+    if (lane == 8) arg = r[8];
+    if (lane == 9) arg = cc[12];
+    const double root = sqrt(arg);
+    auto rootof = [&](int l) { return __shfl_sync(0xffffffffu, root, l); };
+    const double kkt_c = rootof(0);
     // (Halpern iterations: the "average" slot holds T(z) of the last iteration,
     // which is always the candidate)
     const int halp = ctrl->halpern;
-    const double kkt_a = (halp || ctrl->W > 0.0)
-                             ? sqrt(w * w * r[4] + cc[5] / (w * w) + gap_a * gap_a)
-                             : INFINITY;
+    const double root_a = rootof(1);
+    const double kkt_a = (halp || ctrl->W > 0.0) ? root_a : INFINITY;
     const int cand_avg = halp ? 1 : !(kkt_c < kkt_a);
     const double kkt_cand = cand_avg ? kkt_a : kkt_c;
     const double pobj = cand_avg ? pobj_a : pobj_c;
     const double dobj = cand_avg ? dobj_a : dobj_c;
-    const double pres_u = sqrt(cand_avg ? r[5] : r[1]);
-    const double dres_u = sqrt(cand_avg ? cc[6] : cc[1]);
-    const double rel_gap = fabs(dobj - pobj) / (1.0 + fabs(dobj) + fabs(pobj));
-    const double rel_pres = pres_u / (1.0 + ctrl->qnorm);
-    const double rel_dres = dres_u / (1.0 + ctrl->cnorm);
-    const int converged = rel_gap <= ctrl->tol && rel_pres <= ctrl->tol && rel_dres <= ctrl->tol;
-    const int first = ctrl->first;
+    const double p_c = rootof(2), p_a = rootof(3), d_c = rootof(4), d_a = rootof(5);
+    const double pres_u = cand_avg ? p_a : p_c;
+    const double dres_u = cand_avg ? d_a : d_c;
+    const double nx = rootof(6), ny = rootof(7), nadx = rootof(8), nkdy = rootof(9);
     // Algorithm 6 on the last step's differences, as normalised directions:
     // row side r[8] ||A dx||^2, r[9] ||dy||^2, r[10] q^T dy, r[11] max(-G dx), r[12] max(-dy_ineq);
     // column side cc[10] ||dx||^2, cc[11] c^T dx, cc[12] ||K^T dy + dlam||^2, cc[13] ||dlam||^2,
     // cc[14] l^T dlam^+ + u^T dlam^-, cc[15] max distance of dx to V
+    double num = 0.0, den = 1.0;
+    if (lane == 0) num = fabs(dobj - pobj), den = 1.0 + fabs(dobj) + fabs(pobj);
+    if (lane == 1) num = pres_u, den = 1.0 + ctrl->qnorm;
+    if (lane == 2) num = dres_u, den = 1.0 + ctrl->cnorm;
+    if (lane >= 3 && lane < 7) den = nx;
+    if (lane >= 7 && lane < 10) den = ny;
+    if (lane == 3) num = nadx;
+    if (lane == 4) num = -r[11];
+    if (lane == 5) num = cc[11];
+    if (lane == 6) num = cc[15];
+    if (lane == 7) num = nkdy;
+    if (lane == 8) num = -r[12];
+    if (lane == 9) num = r[10] + cc[14];
+    const double quo = num / den;
+    auto quoof = [&](int l) { return __shfl_sync(0xffffffffu, quo, l); };
+    const double rel_gap = quoof(0), rel_pres = quoof(1), rel_dres = quoof(2);
+    const double q3 = quoof(3), q4 = quoof(4), q5 = quoof(5), q6 = quoof(6), q7 = quoof(7),
+                 q8 = quoof(8), q9 = quoof(9);
+    if (lane != 0) return;
+    const int converged = rel_gap <= ctrl->tol && rel_pres <= ctrl->tol && rel_dres <= ctrl->tol;
+    const int first = ctrl->first;
     int infeasible = 0;
     if (!converged && infeas_active(*ctrl)) {
         const double t = ctrl->infeas_tol;
-        const double nx = sqrt(cc[10]), ny = sqrt(r[9] + cc[13]);
-        if (nx > 0.0 && sqrt(r[8]) / nx <= t && -r[11] / nx >= -t && cc[11] / nx <= -t &&
-            cc[15] / nx <= t)
+        if (nx > 0.0 && q3 <= t && q4 >= -t && q5 <= -t && q6 <= t)
             infeasible = LP_DUAL_INFEASIBLE;
-        else if (ny > 0.0 && sqrt(cc[12]) / ny <= t && -r[12] / ny >= -t &&
-                 (r[10] + cc[14]) / ny > t)
+        else if (ny > 0.0 && q7 <= t && q8 >= -t && q9 > t)
             infeasible = LP_PRIMAL_INFEASIBLE;
     }
     int restart = 0;
@@ -291,6 +370,7 @@ __device__ __forceinline__ void check_decide(Ctrl* ctrl, const double* r, const 
         ctrl->kkt_prev = kkt_cand;
         ctrl->fpr_prev = ctrl->fpr;
     }
+    if (omega != w) ctrl->romega = 1.0 / omega;
     ctrl->omega = omega;
     ctrl->restart = restart;
     ctrl->cand_avg = cand_avg;
@@ -335,7 +415,7 @@ __device__ __forceinline__ void check_decide(Ctrl* ctrl, const double* r, const 
     } else if (ctrl->k >= ctrl->max_iters) {
         ctrl->status = LP_ITERATION_LIMIT;
         ctrl->done = 1;
-    } else if ((double)(now - (unsigned long long)ctrl->t0_ns) > ctrl->time_limit_ns) {
+    } else if ((long long)now - ctrl->t0_ns > ctrl->time_limit_ns) {
         ctrl->status = LP_TIME_LIMIT;
         ctrl->done = 1;
     }

@@ -738,6 +738,7 @@ lp_status setup_scale(Handle* h, const lp_opts* o, double* normK)
     k_gather_cast<double><<<grid_for(nnz, 256, 8192), 256, 0, st>>>(nnz, h->tperm, E.val, E.tval);
     ++h->launches;
     LP_CUDA_TRY(cudaGetLastError());
+    LP_TRY(res_values<double>(h));
 
     // Algorithm 2 on K~: b = 1; repeat b <- K~^T (K~ b), b <- b / ||b||; ||K~ b||.
     // The normalisation is carried as a scale of the next K~ product
@@ -750,6 +751,9 @@ lp_status setup_scale(Handle* h, const lp_opts* o, double* normK)
     LP_CUDA_TRY((spmv_prepare<double, EpiStore<double>>()));
     k_fill<double><<<grid_for(n), 256, 0, st>>>(b, n, 1.0);
     ++h->launches;
+    if (E.res.on) {
+        LP_TRY(launch_res_power(h, st, o->power_iters, part + E.npK + 4));
+    } else {
     k_fill<double><<<1, 32, 0, st>>>(inv, 1, 1.0);
     ++h->launches;
     LP_CUDA_TRY(cudaMemsetAsync(go, 0, sizeof(int), st));
@@ -774,6 +778,7 @@ lp_status setup_scale(Handle* h, const lp_opts* o, double* normK)
     ++h->launches;
     k_sum_final<<<1, kCtlNT, 0, st>>>(part, E.npK, part + E.npK + 4);
     ++h->launches;
+    }
     LP_CUDA_TRY(cudaGetLastError());
     double s2 = 0.0;
     int derr = 0;
@@ -937,9 +942,10 @@ lp_status setup_engine(Handle* h, const lp_opts* o)
         T** vm[] = {&E.q,  &E.Y[0], &E.Y[1], &E.KX[0], &E.KX[1],
                     &E.YS, &E.YA,   &E.KXA,  &E.YANC,  &E.KXANC};
         for (T** p : vm) LP_TRY(dev_alloc_n(h, p, (size_t)m));
-        LP_TRY(dev_alloc_n(h, &E.partR, kRowQ * (size_t)kEWGrid));
-        LP_TRY(dev_alloc_n(h, &E.partC, kColQ * (size_t)kEWGrid));
+        LP_TRY(dev_alloc_n(h, &E.partR, kRowQ * (size_t)kCheckGrid));
+        LP_TRY(dev_alloc_n(h, &E.partC, kColQ * (size_t)kCheckGrid));
         LP_TRY(dev_alloc_n(h, &E.ctrl, 1));
+        LP_TRY(res_plan<T>(h));
         E.ready = true;
     }
     if (std::is_same<T, float>::value) {
@@ -958,6 +964,7 @@ lp_status setup_engine(Handle* h, const lp_opts* o)
         k_gather_cast<T><<<grid_for(m), 256, 0, st>>>(m, nullptr, D.q, E.q);
         ++h->launches;
         LP_CUDA_TRY(cudaGetLastError());
+        LP_TRY(res_values<T>(h));
     }
     return LP_OK;
 }

@@ -127,7 +127,7 @@ k_primal_halpern(const Ctrl* __restrict__ ctrl, T* x0, T* x1, const T* __restric
 {
     if (ctrl->skip) return;
     const long long k1 = ctrl->k + 1;
-    const bool hat = k1 % ctrl->check_every == 0 || k1 >= ctrl->max_iters;
+    const bool hat = k1 >= ctrl->next_check || k1 >= ctrl->max_iters;
     T dx2 = T(0);
     using VT = VecTraits<T>;
     constexpr int VEC = VT::N;
@@ -186,15 +186,9 @@ __device__ __noinline__ void decide_thread0(Ctrl* ctrl, bool sums, int adapt, do
     const long long k0 = ctrl->k;
     const double eta = ctrl->eta, omega = ctrl->omega;
     double eta_bar = NAN;
-    if (sums) step_decide(ctrl, adapt, dy2, dx2, inter, &eta_bar);
-    else step_decide(ctrl, adapt, 0.0, 0.0, 0.0);
-    if (ctrl->alog && ctrl->alog_len < ctrl->alog_cap) {
-        double* r = ctrl->alog + kAttemptFields * ctrl->alog_len;
-        r[0] = (double)k0; r[1] = eta; r[2] = eta_bar; r[3] = ctrl->eta;
-        r[4] = ctrl->k != k0 ? 1.0 : 0.0; r[5] = omega;
-        r[6] = sums ? dx2 : NAN; r[7] = sums ? dy2 : NAN; r[8] = sums ? inter : NAN;
-    }
-    ctrl->alog_len += 1;
+    if (sums) step_decide(ctrl, adapt, dy2, dx2, inter, &eta_bar, global_ns());
+    else step_decide(ctrl, adapt, 0.0, 0.0, 0.0, nullptr, global_ns());
+    log_attempt(ctrl, k0, eta, eta_bar, omega, sums, dx2, dy2, inter);
     if (fused) {
         int mode = 0;
         if (!ctrl->done) {
@@ -458,7 +452,7 @@ struct EpiHalpernDual {
         b = sc.hb;
         g = sc.hg;
         const long long k1 = ctrl->k + 1;
-        hat = k1 % ctrl->check_every == 0 || k1 >= ctrl->max_iters;
+        hat = k1 >= ctrl->next_check || k1 >= ctrl->max_iters;
         return true;
     }
     __device__ const T* xin() const { return xh; }
@@ -582,7 +576,7 @@ k_check_prep(const Ctrl* __restrict__ ctrl, const T* x0, const T* x1, const T* y
 // Row side of a KKT check (terms of RowCheck), block partials in FP64:
 // part[q * gridDim.x + block], sums q < kRowSums, then the maxima.
 template <typename T>
-__global__ void __launch_bounds__(kEW)
+__global__ void __launch_bounds__(kCheckNT)
 k_check_rows(const Ctrl* __restrict__ ctrl, const T* y0, const T* y1, const T* kx0,
              const T* kx1, const T* ya, const T* kxa, const T* yanc, const T* q,
              const uint8_t* sense, const T* R, const T* Rinv, int64_t m, double* part)
@@ -595,24 +589,18 @@ k_check_rows(const Ctrl* __restrict__ ctrl, const T* y0, const T* y1, const T* k
     const T* yp = cur ? y0 : y1;
     const T* kxp = cur ? kx0 : kx1;
     RowCheck<T> rc;
-    for (int64_t i = (int64_t)blockIdx.x * kEW + threadIdx.x; i < m; i += (int64_t)gridDim.x * kEW) {
+    for (int64_t i = (int64_t)blockIdx.x * kCheckNT + threadIdx.x; i < m; i += (int64_t)gridDim.x * kCheckNT) {
         const T qi = q[i], ri = Rinv[i], kxi = kx[i], yi = y[i];
         const bool ge = sense[i] != 0;
         rc.add(qi, kxi, yi, kxa[i], ya[i], yanc[i], ri, ge);
         if (inf) rc.add_infeas(qi, kxi, kxp[i], yi, yp[i], R[i], ri, ge);
     }
-    double v[kRowSums], mx[kRowMax];
-#pragma unroll
-    for (int k = 0; k < kRowSums; ++k) v[k] = (double)rc.v[k];
-#pragma unroll
-    for (int k = 0; k < kRowMax; ++k) mx[k] = (double)rc.mx[k];
-    block_partials<kRowSums, kEW>(v, part, gridDim.x);
-    block_partials_max<kRowMax, kEW>(mx, part + (size_t)kRowSums * gridDim.x, gridDim.x);
+    block_check_partials<kRowSums, kRowMax, kCheckNT>(rc.v, rc.mx, part, gridDim.x);
 }
 
 // Column side (terms of ColCheck), same layout with kColSums / kColMax.
 template <typename T>
-__global__ void __launch_bounds__(kEW)
+__global__ void __launch_bounds__(kCheckNT)
 k_check_cols(const Ctrl* __restrict__ ctrl, const T* x0, const T* x1, const T* kty0,
              const T* kty1, const T* xa, const T* ktya, const T* xanc, const T* c,
              const T* l, const T* u, const T* C, const T* Cinv, int64_t n, double* part)
@@ -625,7 +613,7 @@ k_check_cols(const Ctrl* __restrict__ ctrl, const T* x0, const T* x1, const T* k
     const T* xp = cur ? x0 : x1;
     const T* ktyp = cur ? kty0 : kty1;
     ColCheck<T> cc;
-    for (int64_t j = (int64_t)blockIdx.x * kEW + threadIdx.x; j < n; j += (int64_t)gridDim.x * kEW) {
+    for (int64_t j = (int64_t)blockIdx.x * kCheckNT + threadIdx.x; j < n; j += (int64_t)gridDim.x * kCheckNT) {
         const T cj = c[j], lj = l[j], uj = u[j], ci = Cinv[j], xj = x[j], kj = kty[j];
         const T xan = xanc[j];
         const bool lf = isfinite(lj), uf = isfinite(uj);
@@ -633,19 +621,13 @@ k_check_cols(const Ctrl* __restrict__ ctrl, const T* x0, const T* x1, const T* k
         cc.side(1, cj, ktya[j], xa[j], xan, lj, uj, ci, lf, uf);
         if (inf) cc.add_infeas(cj, xj, xp[j], kj, ktyp[j], lj, uj, C[j], ci, lf, uf);
     }
-    double v[kColSums], mx[kColMax];
-#pragma unroll
-    for (int k = 0; k < kColSums; ++k) v[k] = (double)cc.v[k];
-#pragma unroll
-    for (int k = 0; k < kColMax; ++k) mx[k] = (double)cc.mx[k];
-    block_partials<kColSums, kEW>(v, part, gridDim.x);
-    block_partials_max<kColMax, kEW>(mx, part + (size_t)kColSums * gridDim.x, gridDim.x);
+    block_check_partials<kColSums, kColMax, kCheckNT>(cc.v, cc.mx, part, gridDim.x);
 }
 
 // KKT_omega (Section 2.4.2), candidate, termination (Section 2.3.2, unscaled),
 // restart criteria (Section 2.4.2) and Algorithm 4.
 __global__ void __launch_bounds__(kCtlNT)
-k_check_ctrl(Ctrl* ctrl, const double* partR, const double* partC, int nparts,
+k_check_ctrl(Ctrl* ctrl, const double* partR, int nR, const double* partC, int nC,
              lp_trace_rec* trace, double* ftab)
 {
     if (!ctrl->want_check) return;
@@ -673,6 +655,7 @@ k_check_ctrl(Ctrl* ctrl, const double* partR, const double* partC, int nparts,
         const int k = row_side ? q : q - kRowQ;
         const bool is_max = row_side ? k >= kRowSums : k >= kColSums;
         const bool used = inf || (row_side ? k < 8 : k < 10);
+        const int nparts = row_side ? nR : nC;
         const double* part = (row_side ? partR : partC) + (size_t)k * nparts;
         double v = 0.0;
         if (used)
@@ -682,11 +665,7 @@ k_check_ctrl(Ctrl* ctrl, const double* partR, const double* partC, int nparts,
         if (lane == 0) red[q] = v;
     }
     __syncthreads();
-    double r[kRowQ], cc[kColQ];
-    for (int q = 0; q < kRowQ; ++q) r[q] = red[q];
-    for (int q = 0; q < kColQ; ++q) cc[q] = red[kRowQ + q];
-    if (threadIdx.x != 0) return;
-    check_decide(ctrl, r, cc, trace);
+    if (warp == 0) check_decide(ctrl, red, red + kRowQ, trace);
 }
 
 // At a restart the iterate becomes the candidate and the anchor (with its K x);
@@ -809,6 +788,12 @@ static inline int ew_grid(int64_t count)
     return (int)g;
 }
 
+static inline int check_grid(int64_t count)
+{
+    const int64_t g = (count + kCheckNT - 1) / kCheckNT;
+    return (int)(g < 1 ? 1 : g > kCheckGrid ? kCheckGrid : g);
+}
+
 __global__ void k_read_clock(unsigned long long* t) { *t = global_ns(); }
 
 #ifndef PDHG_PRIMAL_GRID
@@ -929,18 +914,29 @@ static void launch_check(Handle* h, Engine<T>& E, cudaStream_t st, cudaGraphCond
     EpiStore<T> e2{E.YA, E.KTYA, nullptr, nullptr, gate};
     launch_spmv<T>(E.gT, st, E.bcol, E.bnzT, E.ntblk, E.wbegT, E.permT, h->trp, h->tci, E.tval, h->dev_err, h->m, e2,
                    false, E.splitT);
-    k_check_rows<T><<<kEWGrid, kEW, 0, st>>>(E.ctrl, E.Y[0], E.Y[1], E.KX[0], E.KX[1], E.YA,
+    k_check_rows<T><<<check_grid(m), kCheckNT, 0, st>>>(E.ctrl, E.Y[0], E.Y[1], E.KX[0], E.KX[1], E.YA,
                                              E.KXA, E.YANC, E.q, h->sense, E.Rt, E.Rinv, m,
                                              E.partR);
-    k_check_cols<T><<<kEWGrid, kEW, 0, st>>>(E.ctrl, E.X[0], E.X[1], E.KTY[0], E.KTY[1], E.XA,
+    k_check_cols<T><<<check_grid(n), kCheckNT, 0, st>>>(E.ctrl, E.X[0], E.X[1], E.KTY[0], E.KTY[1], E.XA,
                                              E.KTYA, E.XANC, E.c, E.l, E.u, E.Ct, E.Cinv, n,
                                              E.partC);
-    k_check_ctrl<<<1, kCtlNT, 0, st>>>(E.ctrl, E.partR, E.partC, kEWGrid, E.trace, E.ftab);
+    k_check_ctrl<<<1, kCtlNT, 0, st>>>(E.ctrl, E.partR, check_grid(m), E.partC, check_grid(n),
+                                       E.trace, E.ftab);
     k_restart_apply<T><<<ew_grid(n + m), kEW, 0, st>>>(
         E.ctrl, E.X[0], E.X[1], E.Y[0], E.Y[1], E.KX[0], E.KX[1], E.KTY[0], E.KTY[1], E.XA, E.YA,
         E.KXA, E.KTYA, E.XANC, E.YANC, E.KXANC, E.XS, E.YS, n, m);
-    if (!halpern) launch_primal<T>(h, E, st);
+    if (!halpern && !E.res.on) launch_primal<T>(h, E, st);
     k_set_cond<<<1, 1, 0, st>>>(E.ctrl, hd, use_handle, in_body);
+}
+
+// The attempts of one loop body: a resident launch (which runs until a check is
+// due), or `slots` attempts.
+template <typename T>
+static lp_status launch_attempts(Handle* h, Engine<T>& E, cudaStream_t st, int slots, bool halpern)
+{
+    if (E.res.on) return launch_res_period<T>(h, st, halpern);
+    for (int s = 0; s < slots; ++s) launch_attempt<T>(h, E, st, halpern);
+    return LP_OK;
 }
 
 template <typename T>
@@ -984,7 +980,7 @@ static lp_status build_graph(Handle* h, Engine<T>& E, int check_every, int slots
     if (conditional) {
         LP_CUDA_TRY(cudaStreamBeginCaptureToGraph(st, body, nullptr, nullptr, 0,
                                                   cudaStreamCaptureModeThreadLocal));
-        for (int s = 0; s < slots; ++s) launch_attempt<T>(h, E, st, halpern != 0);
+        LP_TRY(launch_attempts<T>(h, E, st, slots, halpern != 0));
         launch_check<T>(h, E, st, hd, 1, 1, halpern != 0);
         cudaGraph_t captured = nullptr;
         LP_CUDA_TRY(cudaStreamEndCapture(st, &captured));
@@ -993,7 +989,7 @@ static lp_status build_graph(Handle* h, Engine<T>& E, int check_every, int slots
     } else {
         cudaGraphDestroy(graph);
         LP_CUDA_TRY(cudaStreamBeginCapture(st, cudaStreamCaptureModeThreadLocal));
-        for (int s = 0; s < slots; ++s) launch_attempt<T>(h, E, st, halpern != 0);
+        LP_TRY(launch_attempts<T>(h, E, st, slots, halpern != 0));
         launch_check<T>(h, E, st, hd, 0, 1, halpern != 0);
         cudaGraph_t g2 = nullptr;
         LP_CUDA_TRY(cudaStreamEndCapture(st, &g2));
@@ -1092,7 +1088,7 @@ lp_status run_solve(Handle* h, const lp_opts* o, double eta0, double omega0,
     c.eps_zero = o->eps_zero;
     c.qnorm = h->qnorm;
     c.cnorm = h->cnorm;
-    c.time_limit_ns = o->time_limit_s * 1e9;
+    c.time_limit_ns = limit_ns(o->time_limit_s);
     c.k = k0;
     c.attempts = attempts0;
     c.restarts = restarts0;
@@ -1113,6 +1109,8 @@ lp_status run_solve(Handle* h, const lp_opts* o, double eta0, double omega0,
     c.infeas = o->infeas_detect && !halpern ? 1 : 0;
     c.infeas_tol = o->infeas_tol;
     c.check_every = o->check_every;
+    c.next_check = (k0 / o->check_every + 1) * o->check_every;
+    c.romega = 1.0 / omega0;
     c.px = E.partT;
     c.npx = E.npT;
     refresh_scalars(c);
@@ -1131,7 +1129,7 @@ lp_status run_solve(Handle* h, const lp_opts* o, double eta0, double omega0,
     launch_check<T>(h, E, st, cudaGraphConditionalHandle{}, 0, 0, halpern != 0);
     LP_CUDA_TRY(cudaGetLastError());
     // start state, its two products, the clock read, the start check
-    h->launches += 3 + 1 + check_launches(halpern != 0);
+    h->launches += 3 + 1 + check_launches(halpern != 0 || E.res.on);
 
     const int slots = o->check_every + (c.adaptive ? 4 : 0);
     LP_TRY(build_graph<T>(h, E, o->check_every, slots, o->loop_mode == 1 ? 1 : 0, halpern));
@@ -1149,8 +1147,9 @@ lp_status run_solve(Handle* h, const lp_opts* o, double eta0, double omega0,
         }
     }
     // loop bodies ran on the device: each is `slots` attempts and one check
-    h->launches += out->bodies * (long long)(slots * attempt_launches<T>(halpern != 0) +
-                                             check_launches(halpern != 0));
+    h->launches += out->bodies *
+                   (long long)((E.res.on ? 1 : slots * attempt_launches<T>(halpern != 0)) +
+                               check_launches(halpern != 0 || E.res.on));
     {
         int derr = 0;
         LP_CUDA_TRY(cudaMemcpyAsync(&derr, h->dev_err, sizeof(int), cudaMemcpyDeviceToHost, st));
@@ -1234,7 +1233,8 @@ lp_status profile_step(Handle* h, int reps, double* ms, double* bytes)
     c.done = 0;
     c.max_iters = (long long)1 << 60;
     c.check_every = 1 << 30;
-    c.time_limit_ns = 1e18;
+    c.time_limit_ns = limit_ns(1e9);
+    c.next_check = (long long)1 << 60;
     c.tick = 0;
     c.alog = nullptr;
     LP_CUDA_TRY(cudaMemcpyAsync(E.ctrl, &c, sizeof(Ctrl), cudaMemcpyHostToDevice, st));
