@@ -207,6 +207,19 @@ struct ResPlan {
     unsigned int* seq = nullptr;      // barriers met by earlier launches, arrivals counted
 };
 
+// Sliced rows (sliced.cuh) of one orientation.
+struct SlicedSide {
+    bool on = false;
+    int nslice = 0, grid = 0;
+    int64_t entries = 0;
+    const int4* slice = nullptr;      // first entry / 32, steps, log2 of the lanes per row, first
+                                      // row of the list; the longest first
+    const int32_t* row = nullptr;     // rows of the slices (-1: none)
+    const int32_t* idx = nullptr;     // column of each entry (-1: padding)
+    const int32_t* perm = nullptr;    // its nonzero
+    void* val = nullptr;              // its value
+};
+
 // State and scaled data of one precision T (double or float).
 template <typename T>
 struct Engine {
@@ -238,6 +251,7 @@ struct Engine {
     SchedParams schedK, schedT;                 // parameters of the two schedules
     bool tuned = false;                         // schedules chosen by the autotuner
     ResPlan res;                                // resident iterations (small LPs)
+    SlicedSide slK, slT;                        // sliced rows
     // Ruiz factors R, C and their reciprocals in this precision (KKT checks)
     T* Rt = nullptr; T* Ct = nullptr; T* Rinv = nullptr; T* Cinv = nullptr;
     // reduction partials
@@ -582,6 +596,9 @@ template <typename T> lp_status res_plan(Handle* h);
 template <typename T> lp_status res_values(Handle* h);   // the slices' values from val, tval
 template <typename T> lp_status launch_res_period(Handle* h, cudaStream_t st, bool halpern);
 lp_status launch_res_power(Handle* h, cudaStream_t st, int iters, double* out);
+// sliced.cu: the sliced rows of an engine's sides, and their values from val, tval
+template <typename T> lp_status slice_plan(Handle* h);
+template <typename T> lp_status slice_values(Handle* h);
 // grad.cu
 lp_status run_grad(Handle* h, const lp_opts* o, int K_iters, int ckpt, const double* gxK,
                    double* dc, double* dq, double* dvals, double* xK, int space,

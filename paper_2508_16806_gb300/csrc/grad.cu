@@ -18,7 +18,7 @@
 #include <type_traits>
 
 #include "common.cuh"
-#include "spmv.cuh"
+#include "sliced.cuh"
 
 namespace pdhg {
 
@@ -224,11 +224,9 @@ void forward_step(Handle* h, Engine<T>& E, const double* coef, const T* x, const
     cudaStream_t st = h->stream;
     k_g_primal<T><<<ew_grid_g(h->n), kEW, 0, st>>>(x, kty, E.c, E.l, E.u, coef, xn, mx, h->n);
     EpiGDual<T> ed{xn, y, kx, E.q, h->sense, coef, yn, kxn, my};
-    launch_spmv<T>(E.gK, st, E.brow, E.bnzK, E.nblk, E.wbegK, E.permK, h->rp, h->ci, E.val, h->dev_err, h->n, ed,
-                   false, E.splitK);
+    launch_product<T>(h, E, false, st, ed);
     EpiStore<T> et{yn, ktyn, nullptr, nullptr, nullptr};
-    launch_spmv<T>(E.gT, st, E.bcol, E.bnzT, E.ntblk, E.wbegT, E.permT, h->trp, h->tci, E.tval, h->dev_err, h->m, et,
-                   false, E.splitT);
+    launch_product<T>(h, E, true, st, et);
     h->launches += 3;
 }
 
@@ -237,11 +235,9 @@ lp_status products(Handle* h, Engine<T>& E, const T* x, const T* y, T* kx, T* kt
 {
     cudaStream_t st = h->stream;
     EpiStore<T> e1{x, kx, nullptr, nullptr, nullptr};
-    launch_spmv<T>(E.gK, st, E.brow, E.bnzK, E.nblk, E.wbegK, E.permK, h->rp, h->ci, E.val, h->dev_err, h->n, e1,
-                   false, E.splitK);
+    launch_product<T>(h, E, false, st, e1);
     EpiStore<T> e2{y, kty, nullptr, nullptr, nullptr};
-    launch_spmv<T>(E.gT, st, E.bcol, E.bnzT, E.ntblk, E.wbegT, E.permT, h->trp, h->tci, E.tval, h->dev_err, h->m, e2,
-                   false, E.splitT);
+    launch_product<T>(h, E, true, st, e2);
     h->launches += 2;
     LP_CUDA_TRY(cudaGetLastError());
     return LP_OK;
@@ -374,13 +370,11 @@ lp_status grad_impl(Handle* h, const lp_opts* o, int K, int ckpt, const double* 
             const T* ys = RY + (size_t)s * m;
             k_g_gvy<T><<<ew_grid_g(m), kEW, 0, st>>>(RMY + (size_t)s * m, gy, coef, gvy, ddq, m);
             EpiStore<T> eg{gvy, gxbar, coef + 2, nullptr, nullptr};
-            launch_spmv<T>(E.gT, st, E.bcol, E.bnzT, E.ntblk, E.wbegT, E.permT, h->trp, h->tci, E.tval, h->dev_err,
-                           h->m, eg, false, E.splitT);
+            launch_product<T>(h, E, true, st, eg);
             k_g_gvx<T><<<ew_grid_g(n), kEW, 0, st>>>(RMX + (size_t)s * n, gx, gxbar, coef, gvx, ddc,
                                                     n);
             EpiGy<T> ey{gvx, gvy, coef, gy};
-            launch_spmv<T>(E.gK, st, E.brow, E.bnzK, E.nblk, E.wbegK, E.permK, h->rp, h->ci, E.val, h->dev_err,
-                           h->n, ey, false, E.splitK);
+            launch_product<T>(h, E, false, st, ey);
             if (nnz > 0)
                 k_g_sddmm<T><<<ew_grid_g(nnz), kEW, 0, st>>>(h->krow, h->ci, gvy, gvx, xs, xs1, ys,
                                                              coef, ddv, nnz);

@@ -9,7 +9,7 @@
 #include <type_traits>
 
 #include "common.cuh"
-#include "spmv.cuh"
+#include "sliced.cuh"
 
 namespace pdhg {
 
@@ -739,6 +739,7 @@ lp_status setup_scale(Handle* h, const lp_opts* o, double* normK)
     ++h->launches;
     LP_CUDA_TRY(cudaGetLastError());
     LP_TRY(res_values<double>(h));
+    LP_TRY(slice_values<double>(h));
 
     // Algorithm 2 on K~: b = 1; repeat b <- K~^T (K~ b), b <- b / ||b||; ||K~ b||.
     // The normalisation is carried as a scale of the next K~ product
@@ -761,20 +762,17 @@ lp_status setup_scale(Handle* h, const lp_opts* o, double* normK)
     ++h->launches;
     for (int it = 0; it < o->power_iters; ++it) {
         EpiStore<double> e1{b, t, inv, nullptr, go};
-        launch_spmv<double>(E.gK, st, E.brow, E.bnzK, E.nblk, E.wbegK, E.permK, h->rp, h->ci, E.val, h->dev_err, h->n, e1,
-                            false, E.splitK);
+        launch_product<double>(h, E, false, st, e1);
         ++h->launches;
         EpiStore<double> e2{t, b, nullptr, part, go};
-        launch_spmv<double>(E.gT, st, E.bcol, E.bnzT, E.ntblk, E.wbegT, E.permT, h->trp, h->tci, E.tval, h->dev_err, h->m,
-                            e2, false, E.splitT);
+        launch_product<double>(h, E, true, st, e2);
         ++h->launches;
         k_pow_inv_norm<<<1, kCtlNT, 0, st>>>(part, E.npT, inv, go);
         ++h->launches;
         LP_CUDA_TRY(cudaGetLastError());
     }
     EpiStore<double> e3{b, t, inv, part, nullptr};
-    launch_spmv<double>(E.gK, st, E.brow, E.bnzK, E.nblk, E.wbegK, E.permK, h->rp, h->ci, E.val, h->dev_err, h->n, e3,
-                        false, E.splitK);
+    launch_product<double>(h, E, false, st, e3);
     ++h->launches;
     k_sum_final<<<1, kCtlNT, 0, st>>>(part, E.npK, part + E.npK + 4);
     ++h->launches;
@@ -816,6 +814,34 @@ static lp_status upload_split(Handle* h, const SplitPlan& plan, SplitRows& sp)
     sp.info = info;
     sp.slots = slots;
     sp.n = plan.n;
+    return LP_OK;
+}
+
+// A side in sliced rows: its launch's blocks and partials.
+template <typename T>
+static lp_status engine_grids(Handle* h, Engine<T>& E)
+{
+    if (E.slK.on) {
+        E.gK = E.npK = E.slK.grid;
+        E.splitK.n = 0;
+    }
+    if (E.slT.on) {
+        E.gT = E.npT = E.slT.grid;
+        E.splitT.n = 0;
+    }
+    const size_t needD = 2 * (size_t)E.npK + 8, needT = std::max<size_t>((size_t)E.npT, (size_t)kEWGrid) + 8;
+    if (needD > E.partD_cap) {
+        dev_free(h, E.partD);
+        E.partD = nullptr;
+        LP_TRY(dev_alloc_n(h, &E.partD, needD));
+        E.partD_cap = needD;
+    }
+    if (needT > E.partT_cap) {
+        dev_free(h, E.partT);
+        E.partT = nullptr;
+        LP_TRY(dev_alloc_n(h, &E.partT, needT));
+        E.partT_cap = needT;
+    }
     return LP_OK;
 }
 
@@ -867,22 +893,8 @@ lp_status engine_schedule(Handle* h, SchedParams sK, SchedParams sT)
     for (size_t t = 0; t < spT.task_piece.size(); ++t)
         if (spT.task_piece[t] >= 0) nt[t] |= (int64_t)(spT.task_piece[t] + 1) << 32;
     // step partials: one per block, then one per split row
-    const size_t npK = (size_t)gK + (size_t)spK.n, npT = (size_t)gT + (size_t)spT.n;
-    const size_t needD = 2 * npK + 8, needT = std::max<size_t>(npT, (size_t)kEWGrid) + 8;
-    if (needD > E.partD_cap) {
-        dev_free(h, E.partD);
-        E.partD = nullptr;
-        LP_TRY(dev_alloc_n(h, &E.partD, needD));
-        E.partD_cap = needD;
-    }
-    if (needT > E.partT_cap) {
-        dev_free(h, E.partT);
-        E.partT = nullptr;
-        LP_TRY(dev_alloc_n(h, &E.partT, needT));
-        E.partT_cap = needT;
-    }
-    E.npK = (int)npK;
-    E.npT = (int)npT;
+    E.npK = gK + spK.n;
+    E.npT = gT + spT.n;
     LP_TRY(dev_alloc_n(h, &E.brow, bk.size()));
     LP_TRY(dev_alloc_n(h, &E.bcol, bt.size()));
     LP_TRY(dev_alloc_n(h, &E.bnzK, nk.size()));
@@ -914,6 +926,7 @@ lp_status engine_schedule(Handle* h, SchedParams sK, SchedParams sT)
     E.ntblk = (int)bt.size() - 1;
     E.gK = gK;
     E.gT = gT;
+    LP_TRY(engine_grids(h, E));
     E.schedK = sK;
     E.schedT = sT;
     return LP_OK;
@@ -946,6 +959,8 @@ lp_status setup_engine(Handle* h, const lp_opts* o)
         LP_TRY(dev_alloc_n(h, &E.partC, kColQ * (size_t)kCheckGrid));
         LP_TRY(dev_alloc_n(h, &E.ctrl, 1));
         LP_TRY(res_plan<T>(h));
+        if (!E.res.on) LP_TRY(slice_plan<T>(h));
+        LP_TRY(engine_grids(h, E));
         E.ready = true;
     }
     if (std::is_same<T, float>::value) {
@@ -965,6 +980,7 @@ lp_status setup_engine(Handle* h, const lp_opts* o)
         ++h->launches;
         LP_CUDA_TRY(cudaGetLastError());
         LP_TRY(res_values<T>(h));
+        LP_TRY(slice_values<T>(h));
     }
     return LP_OK;
 }

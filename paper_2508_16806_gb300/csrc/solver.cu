@@ -39,7 +39,7 @@
 
 #include "common.cuh"
 #include "control.cuh"
-#include "spmv.cuh"
+#include "sliced.cuh"
 
 namespace pdhg {
 
@@ -837,8 +837,7 @@ static void launch_dual(Handle* h, Engine<T>& E, cudaStream_t st)
 {
     EpiDual<T> ed{E.ctrl, E.X[0], E.X[1], E.Y[0], E.Y[1], E.KX[0], E.KX[1], E.YS, E.q, h->sense,
                   E.partD};
-    launch_spmv<T>(E.gK, st, E.brow, E.bnzK, E.nblk, E.wbegK, E.permK, h->rp, h->ci, E.val, h->dev_err, h->n, ed,
-                   true, E.splitK);
+    launch_product<T>(h, E, false, st, ed, true);
 }
 
 template <typename T>
@@ -847,8 +846,7 @@ static void launch_primal_step(Handle* h, Engine<T>& E, cudaStream_t st, bool wi
     constexpr bool F = FusePrimal<T>::value;
     EpiPrimalStep<T, F> ep{E.ctrl, E.X[0], E.X[1], E.Y[0], E.Y[1], E.KTY[0], E.KTY[1], E.c, E.l,
                            E.u, E.XS, E.partT, h->n};
-    launch_spmv<T>(E.gT, st, E.bcol, E.bnzT, E.ntblk, E.wbegT, E.permT, h->trp, h->tci, E.tval,
-                   h->dev_err, h->m, ep, true, E.splitT);
+    launch_product<T>(h, E, true, st, ep, true);
     if (!F && with_primal) launch_primal<T>(h, E, st, 1);
 }
 
@@ -858,8 +856,7 @@ static void launch_primal_t(Handle* h, Engine<T>& E, cudaStream_t st)
 {
     EpiPrimalT<T> et{E.ctrl, E.Y[0], E.Y[1], E.KTY[0], E.KTY[1], E.partT, primal_grid<T>(h->n),
                      E.partD, E.npK};
-    launch_spmv<T>(E.gT, st, E.bcol, E.bnzT, E.ntblk, E.wbegT, E.permT, h->trp, h->tci, E.tval, h->dev_err, h->m, et,
-                   false, E.splitT);
+    launch_product<T>(h, E, true, st, et);
 }
 
 template <typename T>
@@ -875,8 +872,7 @@ static void launch_dual_halpern(Handle* h, Engine<T>& E, cudaStream_t st)
 {
     EpiHalpernDual<T> ed{E.ctrl, E.XH, E.Y[0], E.Y[1], E.KX[0], E.KX[1], E.YANC, E.KXANC, E.YA,
                          E.q, h->sense, E.partD};
-    launch_spmv<T>(E.gK, st, E.brow, E.bnzK, E.nblk, E.wbegK, E.permK, h->rp, h->ci, E.val,
-                   h->dev_err, h->n, ed, false, E.splitK);
+    launch_product<T>(h, E, false, st, ed);
 }
 
 // one step attempt: 2 launches (PDHG) or 3 (a Halpern iteration)
@@ -909,11 +905,9 @@ static void launch_check(Handle* h, Engine<T>& E, cudaStream_t st, cudaGraphCond
                                                      E.YS, E.XA, E.YA, E.l, E.u, h->sense, n, m);
     const int* gate = &E.ctrl->want_check;
     EpiStore<T> e1{E.XA, E.KXA, nullptr, nullptr, gate};
-    launch_spmv<T>(E.gK, st, E.brow, E.bnzK, E.nblk, E.wbegK, E.permK, h->rp, h->ci, E.val, h->dev_err, h->n, e1,
-                   false, E.splitK);
+    launch_product<T>(h, E, false, st, e1);
     EpiStore<T> e2{E.YA, E.KTYA, nullptr, nullptr, gate};
-    launch_spmv<T>(E.gT, st, E.bcol, E.bnzT, E.ntblk, E.wbegT, E.permT, h->trp, h->tci, E.tval, h->dev_err, h->m, e2,
-                   false, E.splitT);
+    launch_product<T>(h, E, true, st, e2);
     k_check_rows<T><<<check_grid(m), kCheckNT, 0, st>>>(E.ctrl, E.Y[0], E.Y[1], E.KX[0], E.KX[1], E.YA,
                                              E.KXA, E.YANC, E.q, h->sense, E.Rt, E.Rinv, m,
                                              E.partR);
@@ -1041,11 +1035,9 @@ lp_status run_solve(Handle* h, const lp_opts* o, double eta0, double omega0,
                                                      E.l, E.u, h->sense, h->R, h->C, wxs, wys,
                                                      dwx, dwy, n, m);
     EpiStore<T> e1{E.X[0], E.KX[0], nullptr, nullptr, nullptr};
-    launch_spmv<T>(E.gK, st, E.brow, E.bnzK, E.nblk, E.wbegK, E.permK, h->rp, h->ci, E.val, h->dev_err, h->n, e1,
-                   false, E.splitK);
+    launch_product<T>(h, E, false, st, e1);
     EpiStore<T> e2{E.Y[0], E.KTY[0], nullptr, nullptr, nullptr};
-    launch_spmv<T>(E.gT, st, E.bcol, E.bnzT, E.ntblk, E.wbegT, E.permT, h->trp, h->tci, E.tval, h->dev_err, h->m, e2,
-                   false, E.splitT);
+    launch_product<T>(h, E, true, st, e2);
     LP_CUDA_TRY(cudaGetLastError());
     if (m > 0)
         LP_CUDA_TRY(cudaMemcpyAsync(E.KXANC, E.KX[0], sizeof(T) * m, cudaMemcpyDeviceToDevice, st));
