@@ -136,47 +136,6 @@ __global__ void k_lp_sumsq(const double* v, const int64_t* off, double* out)
     }
 }
 
-// ---------------------------------------------------------------- Ruiz per LP
-
-// per-LP deviation max |1 - norm| (bit pattern max) of non-empty rows / columns
-__global__ void k_ruiz_dev_lp(int64_t m, int64_t n, const double* rn, const double* cn,
-                              const int32_t* lp_row, const int32_t* lp_col,
-                              unsigned long long* dev)
-{
-    for (int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; t < m + n;
-         t += (int64_t)gridDim.x * blockDim.x) {
-        const double v = t < m ? rn[t] : cn[t - m];
-        const int k = t < m ? lp_row[t] : lp_col[t - m];
-        if (v > 0.0)
-            atomicMax(dev + k, (unsigned long long)__double_as_longlong(fabs(1.0 - v)));
-    }
-}
-
-// LPs whose deviation is within tol stop (sticky); returns the count still going
-__global__ void k_ruiz_stop_lp(int B, const unsigned long long* dev, double tol, int* go,
-                               int* live)
-{
-    for (int k = threadIdx.x; k < B; k += blockDim.x) {
-        double d;
-        const unsigned long long b = dev[k];
-        memcpy(&d, &b, sizeof(d));
-        if (go[k] && d <= tol) go[k] = 0;
-        if (go[k]) atomicAdd(live, 1);
-    }
-}
-
-// factor 1/sqrt(norm) for a going LP, 1 otherwise (and for empty rows / columns)
-__global__ void k_ruiz_factors_lp(int64_t count, double* nrm, double* acc, const int32_t* lp,
-                                  const int* go)
-{
-    for (int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; t < count;
-         t += (int64_t)gridDim.x * blockDim.x) {
-        const double f = (go[lp[t]] && nrm[t] > 0.0) ? 1.0 / sqrt(nrm[t]) : 1.0;
-        nrm[t] = f;
-        acc[t] *= f;
-    }
-}
-
 // ---------------------------------------------------------------- per-task epilogues
 
 // out[r] = v; per-task partial of sum out^2 (power iteration); gated per LP
@@ -872,47 +831,24 @@ lp_status batch_scale(BatchHandle* bh, const lp_opts* o, double* normK_dev)
                                 cudaMemcpyDeviceToDevice, st));
     // tuned before the power iteration uses it (same order of sums in every solve)
     if (o->autotune) LP_TRY(tune_batch<double>(bh));
-    k_fill_f64<<<grid_n(m, 256, 65535), 256, 0, st>>>(h->R, m, 1.0);
-    k_fill_f64<<<grid_n(n, 256, 65535), 256, 0, st>>>(h->C, n, 1.0);
+    kb_cast<double><<<grid_n(nnz, 256, 8192), 256, 0, st>>>(E.val, h->tperm, E.tval, nnz);
+    ++h->launches;
+    LP_TRY(ruiz_scale(h, o->ruiz_iters, o->ruiz_tol, E.val, E.tval, B, bh->meta.lp_row, bh->meta.lp_col,
+                      reinterpret_cast<unsigned long long*>(bh->lpd)));
     double* rn = h->scratch;
     double* cn = h->scratch + m;
-    unsigned long long* dev = reinterpret_cast<unsigned long long*>(bh->lpd);
-    int* live = reinterpret_cast<int*>(bh->lpd + B);
-    k_fill_i32<<<grid_n(B, 256, 4096), 256, 0, st>>>(reinterpret_cast<int32_t*>(bh->go), B, 1);
-    for (int it = 0; it < o->ruiz_iters; ++it) {
-        k_row_inf<<<grid_n(m * 32, 256, 65535 * 8), 256, 0, st>>>(m, h->rp, E.val, rn);
-        LP_CUDA_TRY(cudaMemsetAsync(cn, 0, sizeof(double) * (size_t)n, st));
-        k_col_inf<<<grid_n(nnz, 256, 8192), 256, 0, st>>>(
-            nnz, h->ci, E.val, reinterpret_cast<unsigned long long*>(cn));
-        LP_CUDA_TRY(cudaMemsetAsync(dev, 0, sizeof(unsigned long long) * B, st));
-        k_ruiz_dev_lp<<<grid_n(m + n, 256, 4096), 256, 0, st>>>(m, n, rn, cn, bh->meta.lp_row,
-                                                                bh->meta.lp_col, dev);
-        LP_CUDA_TRY(cudaMemsetAsync(live, 0, sizeof(int), st));
-        k_ruiz_stop_lp<<<1, 256, 0, st>>>(B, dev, o->ruiz_tol, bh->go, live);
-        int hl = 0;
-        LP_CUDA_TRY(cudaMemcpyAsync(&hl, live, sizeof(int), cudaMemcpyDeviceToHost, st));
-        LP_CUDA_TRY(cudaStreamSynchronize(st));
-        if (hl == 0) break;
-        k_ruiz_factors_lp<<<grid_n(m, 256, 65535), 256, 0, st>>>(m, rn, h->R, bh->meta.lp_row,
-                                                                 bh->go);
-        k_ruiz_factors_lp<<<grid_n(n, 256, 65535), 256, 0, st>>>(n, cn, h->C, bh->meta.lp_col,
-                                                                 bh->go);
-        k_scale_vals<<<grid_n(nnz, 256, 8192), 256, 0, st>>>(nnz, h->krow, h->ci, rn, cn, E.val);
-        h->launches += 7;
-        LP_CUDA_TRY(cudaGetLastError());
-    }
     if (o->pock_chambolle) {
         k_pc_sums<<<grid_n(m + n, 256, 65535), 256, 0, st>>>(m, n, h->rp, h->trp, h->tperm, E.val,
                                                              o->pc_alpha, rn, cn);
         k_ruiz_factors<<<grid_n(m, 256, 65535), 256, 0, st>>>(m, rn, h->R);
         k_ruiz_factors<<<grid_n(n, 256, 65535), 256, 0, st>>>(n, cn, h->C);
         k_scale_vals<<<grid_n(nnz, 256, 8192), 256, 0, st>>>(nnz, h->krow, h->ci, rn, cn, E.val);
-        h->launches += 4;
+        kb_cast<double><<<grid_n(nnz, 256, 8192), 256, 0, st>>>(E.val, h->tperm, E.tval, nnz);
+        h->launches += 5;
     }
     k_scale_vectors<<<grid_n(m + n, 256, 65535), 256, 0, st>>>(m, n, h->R, h->C, h->c0, h->q0,
                                                                h->l0, h->u0, E.c, E.q, E.l, E.u);
-    kb_cast<double><<<grid_n(nnz, 256, 8192), 256, 0, st>>>(E.val, h->tperm, E.tval, nnz);
-    h->launches += 2;
+    ++h->launches;
     LP_CUDA_TRY(cudaGetLastError());
     // Algorithm 2 per LP
     LP_CUDA_TRY((spmv_prepare<double, EpiBStore<double>>()));

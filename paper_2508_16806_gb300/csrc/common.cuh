@@ -546,8 +546,20 @@ __device__ __forceinline__ unsigned long long global_ns()
 
 // ------------------------------------------------------------ setup kernels
 // (defined in setup.cu; the batched solver launches them too)
-__global__ void k_row_inf(int64_t m, const int64_t* rp, const double* v, double* rn);
-__global__ void k_col_inf(int64_t nnz, const int32_t* ci, const double* v, unsigned long long* cn);
+constexpr int kRuizNT = 256;
+// one side of a Ruiz pass: K (rows) or K^T (columns)
+struct RuizSide {
+    int64_t rows, chunk;            // chunk: rows of a block
+    const int64_t* rp;
+    const int32_t* ci;
+    double* v;
+    const double *own, *other;      // factors of this side's rows / of the other side's
+    double* nrm;
+    const int32_t* lp;              // the LP of a row, or nullptr
+    int lg, blocks;                 // log2 of the lanes per row
+};
+lp_status ruiz_scale(Handle* h, int iters, double tol, double* val, double* tval, int B,
+                     const int32_t* lp_row, const int32_t* lp_col, unsigned long long* dev);
 __global__ void k_ruiz_factors(int64_t count, double* nrm, double* acc);
 __global__ void k_scale_vals(int64_t nnz, const int32_t* krow, const int32_t* ci, const double* r,
                              const double* s, double* v);

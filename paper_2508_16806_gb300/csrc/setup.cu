@@ -345,45 +345,184 @@ __global__ void k_fill(T* p, int64_t count, T v)
         p[t] = v;
 }
 
-// Ruiz: row infinity norms (one warp per row, exact max)
-__global__ void k_row_inf(int64_t m, const int64_t* rp, const double* v, double* rn)
+// One Ruiz pass over both sides of the matrix (blocks [0, a.blocks): rows of K, the rest:
+// rows of K^T).  SCALE: the entries take the factors of the previous pass, in the same
+// order of products on both sides, so K^T stays the exact transpose of K.  NORMS: infinity
+// norms of the rows and their largest deviation |1 - norm| (non-empty rows) per LP.
+// Groups of 2^lg lanes take a row, four entries per lane in flight (past the end: the
+// lane's first entry again), the whole warp what is left of a row after 16 entries per lane.  Both sides hold their values, so no norm needs an atomic per
+// nonzero and no pass reads the matrix a second time; the maxima are of bit patterns (they
+// order like the non-negative values: an FP64 maximum costs 200 cycles of a warp here).
+// Bound by the chain of a row's loads (start, entries, factors).  64 LPs stacked: the passes
+// of a solve, with an atomic per nonzero for the column norms (a warp per row 417 us) and
+// one per row for the deviation (902 us a pass), 14 -> 2 ms, a solve 58.2 -> 46.5 ms.  1M x
+// 2M LP with 20M power-law rows: 647 us a pass (830 us with lanes chosen for the longest row).
+template <bool SCALE, bool NORMS>
+__global__ void __launch_bounds__(kRuizNT)
+k_ruiz_pass(RuizSide a, RuizSide b, unsigned long long* dev)
 {
+    __shared__ unsigned long long shd[kRuizNT / 32];
+    __shared__ int shk[kRuizNT / 32];
+    const bool tside = (int)blockIdx.x >= a.blocks;
+    const RuizSide S = tside ? b : a;
+    const int lg = S.lg, G = 1 << lg, per = kRuizNT >> lg;
+    const int g = threadIdx.x & (G - 1);
+    const int64_t r0 = (int64_t)(blockIdx.x - (tside ? a.blocks : 0)) * S.chunk;
+    const int64_t r1 = r0 + S.chunk < S.rows ? r0 + S.chunk : S.rows;
     const int lane = threadIdx.x & 31;
-    const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
-    // the trip count is uniform per warp (w steps by whole warps)
-    for (int64_t w = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; w < m; w += nw) {
-        double a = 0.0;
-        for (int64_t p = rp[w] + lane; p < rp[w + 1]; p += 32) a = fmax(a, fabs(v[p]));
+    int kc = 0;
+    unsigned long long dm = 0;
+    // entries p, p + w, p + 2 w, p + 3 w below e (p is): largest magnitude, as bits
+    const auto take = [&](int64_t p, int64_t e, int w, double own) {
+        int64_t q[4];
+        double v[4], f[4];
+        int c[4];
+        unsigned long long mx = 0;
 #pragma unroll
-        for (int o = 16; o > 0; o >>= 1) a = fmax(a, __shfl_down_sync(0xffffffffu, a, o));
-        if (lane == 0) rn[w] = a;
+        for (int u = 0; u < 4; ++u) q[u] = p + u * w < e ? p + u * w : p;
+#pragma unroll
+        for (int u = 0; u < 4; ++u) v[u] = S.v[q[u]];
+        if (SCALE) {
+#pragma unroll
+            for (int u = 0; u < 4; ++u) c[u] = S.ci[q[u]];
+#pragma unroll
+            for (int u = 0; u < 4; ++u) f[u] = S.other[c[u]];
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+                const double x = v[u] * (tside ? f[u] : own);
+                v[u] = x * (tside ? own : f[u]);
+                if (p + u * w < e) S.v[q[u]] = v[u];
+            }
+        }
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+            const unsigned long long t = (unsigned long long)__double_as_longlong(fabs(v[u]));
+            mx = t > mx ? t : mx;
+        }
+        return mx;
+    };
+    // the row of the next round is fetched a round ahead
+    int64_t row = r0 + (threadIdx.x >> lg), pn = 0, en = 0;
+    double on = 1.0;
+    if (row < r1) {
+        pn = S.rp[row];
+        en = S.rp[row + 1];
+        if (SCALE) on = S.own[row];
+    }
+    for (int64_t base = r0; base < r1; base += per, row += per) {
+        const bool in = row < r1;
+        int64_t p = pn + g;
+        const int64_t e = en;
+        const double own = on;
+        pn = en = 0;
+        if (row + per < r1) {
+            pn = S.rp[row + per];
+            en = S.rp[row + per + 1];
+            if (SCALE) on = S.own[row + per];
+        }
+        unsigned long long mx = 0;
+        for (int k = 0; k < 4 && p < e; ++k, p += 4 * G) {
+            const unsigned long long t = take(p, e, G, own);
+            mx = t > mx ? t : mx;
+        }
+        // what is left of long rows: by the whole warp, one row after the other
+        unsigned rest = __ballot_sync(0xffffffffu, g == 0 && p < e);
+        for (; rest; rest &= rest - 1) {
+            const int src = __ffs(rest) - 1;
+            const int64_t p0 = __shfl_sync(0xffffffffu, p, src), e0 = __shfl_sync(0xffffffffu, e, src);
+            const double o0 = __shfl_sync(0xffffffffu, own, src);
+            unsigned long long t = 0;
+            for (int64_t pp = p0 + lane; pp < e0; pp += 128) {
+                const unsigned long long t1 = take(pp, e0, 32, o0);
+                t = t1 > t ? t1 : t;
+            }
+            for (int o = 16; o > 0; o >>= 1) {
+                const unsigned long long t1 = __shfl_xor_sync(0xffffffffu, t, o);
+                t = t1 > t ? t1 : t;
+            }
+            if (lane == src) mx = t > mx ? t : mx;
+        }
+        if (NORMS) {
+            for (int o = G >> 1; o > 0; o >>= 1) {
+                const unsigned long long t = __shfl_xor_sync(0xffffffffu, mx, o);
+                mx = t > mx ? t : mx;
+            }
+            if (in) {
+                const double nr = __longlong_as_double((long long)mx);
+                if (g == 0) S.nrm[row] = nr;
+                const int k = S.lp ? S.lp[row] : 0;
+                if (k != kc) {
+                    if (g == 0 && dm) atomicMax(dev + kc, dm);
+                    kc = k;
+                    dm = 0;
+                }
+                const unsigned long long t = (unsigned long long)__double_as_longlong(fabs(1.0 - nr));
+                if (mx != 0 && t > dm) dm = t;
+            }
+        }
+    }
+    if (NORMS) {
+        int same = 0;
+        __match_all_sync(0xffffffffu, kc, &same);
+        if (!same && g == 0 && dm) atomicMax(dev + kc, dm);
+        for (int o = 16; o > 0; o >>= 1) {
+            const unsigned long long t = __shfl_xor_sync(0xffffffffu, dm, o);
+            dm = t > dm ? t : dm;
+        }
+        if ((threadIdx.x & 31) == 0) {
+            shd[threadIdx.x >> 5] = same ? dm : 0;
+            shk[threadIdx.x >> 5] = kc;
+        }
+        __syncthreads();
+        if (threadIdx.x == 0) {
+            kc = shk[0];
+            dm = shd[0];
+            for (int w = 1; w < kRuizNT / 32; ++w) {
+                if (shk[w] != kc) {
+                    if (dm) atomicMax(dev + kc, dm);
+                    kc = shk[w];
+                    dm = 0;
+                }
+                dm = shd[w] > dm ? shd[w] : dm;
+            }
+            if (dm) atomicMax(dev + kc, dm);
+        }
     }
 }
 
-// Ruiz: column infinity norms by an integer max on the bit pattern
-// (non-negative IEEE doubles order like their bits).
-__global__ void k_col_inf(int64_t nnz, const int32_t* ci, const double* v, unsigned long long* cn)
+// Factors of the next pass: 1 / sqrt(norm), or 1 for an empty row or column and for an
+// LP whose deviation is within tol (its entries no longer change, so neither does its
+// deviation: it has stopped for good).  dev_next is cleared for the next pass.
+__global__ void k_ruiz_next(int64_t m, int64_t n, const double* nrm, double* fac, double* R, double* C,
+                            const int32_t* lp_row, const int32_t* lp_col,
+                            const unsigned long long* dev, unsigned long long* dev_next, int B,
+                            double tol)
 {
-    for (int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; p < nnz;
-         p += (int64_t)gridDim.x * blockDim.x) {
-        const double a = fabs(v[p]);
-        atomicMax(cn + ci[p], (unsigned long long)__double_as_longlong(a));
-    }
-}
-
-// deviation max |1 - norm| over non-empty rows and columns -> dev (bit pattern max)
-__global__ void k_ruiz_dev(int64_t m, int64_t n, const double* rn, const double* cn,
-                           unsigned long long* dev)
-{
-    double d = 0.0;
+    if (blockIdx.x == 0)
+        for (int k = threadIdx.x; k < B; k += blockDim.x) dev_next[k] = 0;
     for (int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; t < m + n;
          t += (int64_t)gridDim.x * blockDim.x) {
-        const double v = t < m ? rn[t] : cn[t - m];
-        if (v > 0.0) d = fmax(d, fabs(1.0 - v));
+        const bool row = t < m;
+        const int k = lp_row ? (row ? lp_row[t] : lp_col[t - m]) : 0;
+        const bool stop = __longlong_as_double((long long)dev[k]) <= tol;
+        const double v = nrm[t];
+        const double f = !stop && v > 0.0 ? 1.0 / sqrt(v) : 1.0;
+        fac[t] = f;
+        double* acc = row ? R + t : C + (t - m);
+        *acc *= f;
     }
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) d = fmax(d, __shfl_down_sync(0xffffffffu, d, o));
-    if ((threadIdx.x & 31) == 0) atomicMax(dev, (unsigned long long)__double_as_longlong(d));
+}
+
+// LPs whose deviation is still above tol
+__global__ void k_ruiz_live(int B, const unsigned long long* dev, double tol, int* live)
+{
+    __shared__ int n;
+    if (threadIdx.x == 0) n = 0;
+    __syncthreads();
+    for (int k = threadIdx.x; k < B; k += blockDim.x)
+        if (!(__longlong_as_double((long long)dev[k]) <= tol)) atomicAdd(&n, 1);
+    __syncthreads();
+    if (threadIdx.x == 0) *live = n;
 }
 
 // norm -> factor 1/sqrt(norm) (1 for an empty row/column); accumulate
@@ -678,6 +817,61 @@ lp_status setup_update(Handle* h, const double* vals, const double* c, const dou
     return LP_OK;
 }
 
+// Algorithm 3 in place on val / tval (tval: the transpose of val), accumulated into R and C
+// (set to 1 here).  B LPs of the stacked matrix (lp_row, lp_col: the LP of a row / column; a
+// single LP: nullptr); dev: 2 B + 1 scratch words.  The host looks whether all LPs have
+// stopped after every fourth pass only: passes past the end multiply by one.
+lp_status ruiz_scale(Handle* h, int iters, double tol, double* val, double* tval, int B,
+                     const int32_t* lp_row, const int32_t* lp_col, unsigned long long* dev)
+{
+    const int64_t m = h->m, n = h->n;
+    cudaStream_t st = h->stream;
+    double* fac = h->scratch;
+    double* nrm = h->scratch + m + n;
+    k_fill<double><<<grid_for(m), 256, 0, st>>>(h->R, m, 1.0);
+    k_fill<double><<<grid_for(n), 256, 0, st>>>(h->C, n, 1.0);
+    h->launches += 2;
+    if (iters <= 0) return LP_OK;
+    int sms = 0;
+    LP_CUDA_TRY(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, h->device));
+    const auto side = [&](int64_t rows, const int64_t* rp, const int32_t* ci, double* v,
+                          const double* own, const double* other, double* nr, const int32_t* lp) {
+        // lanes per row: the average row in one go of four entries a lane
+        int lg = 0;
+        while (lg < 5 && (rows << (lg + 2)) < h->nnz) ++lg;
+        const int64_t per = kRuizNT >> lg, blocks = std::min<int64_t>((rows + per - 1) / per, 16 * sms);
+        const int64_t chunk = (((rows + blocks - 1) / blocks) + per - 1) / per * per;
+        return RuizSide{rows, chunk, rp, ci, v, own, other, nr, lp, lg, (int)((rows + chunk - 1) / chunk)};
+    };
+    const RuizSide a = side(m, h->rp, h->ci, val, fac, fac + m, nrm, lp_row);
+    const RuizSide b = side(n, h->trp, h->tci, tval, fac + m, fac, nrm + m, lp_col);
+    const int grid = a.blocks + b.blocks;
+    int* live = reinterpret_cast<int*>(dev + 2 * B);
+    LP_CUDA_TRY(cudaMemsetAsync(dev, 0, sizeof(unsigned long long) * 2 * (size_t)B, st));
+    for (int it = 0; it < iters; ++it) {
+        unsigned long long *d = dev + (it & 1) * B, *dn = dev + ((it + 1) & 1) * B;
+        if (it == 0)
+            k_ruiz_pass<false, true><<<grid, kRuizNT, 0, st>>>(a, b, d);
+        else
+            k_ruiz_pass<true, true><<<grid, kRuizNT, 0, st>>>(a, b, d);
+        k_ruiz_next<<<grid_for(m + n), 256, 0, st>>>(m, n, nrm, fac, h->R, h->C, lp_row, lp_col, d, dn, B,
+                                                     tol);
+        h->launches += 2;
+        if (it % 4 == 3 && it + 1 < iters) {
+            int hl = 0;
+            k_ruiz_live<<<1, 256, 0, st>>>(B, d, tol, live);
+            ++h->launches;
+            LP_CUDA_TRY(cudaMemcpyAsync(&hl, live, sizeof(int), cudaMemcpyDeviceToHost, st));
+            LP_CUDA_TRY(cudaStreamSynchronize(st));
+            if (hl == 0) break;
+        }
+    }
+    k_ruiz_pass<true, false><<<grid, kRuizNT, 0, st>>>(a, b, dev);
+    ++h->launches;
+    LP_CUDA_TRY(cudaGetLastError());
+    return LP_OK;
+}
+
 // Algorithm 3 (+ optional Pock-Chambolle) into e64.val and R, C, the scaled
 // vectors e64.c/q/l/u and the scaled transpose e64.tval; then Algorithm 2.
 lp_status setup_scale(Handle* h, const lp_opts* o, double* normK)
@@ -687,38 +881,13 @@ lp_status setup_scale(Handle* h, const lp_opts* o, double* normK)
     cudaStream_t st = h->stream;
     LP_CUDA_TRY(cudaMemcpyAsync(E.val, h->val0, pad8(nnz) * sizeof(double),
                                 cudaMemcpyDeviceToDevice, st));
-    k_fill<double><<<grid_for(m), 256, 0, st>>>(h->R, m, 1.0);
+    LP_CUDA_TRY(cudaMemsetAsync(E.tval, 0, pad8(nnz) * sizeof(double), st));
+    k_gather_cast<double><<<grid_for(nnz, 256, 8192), 256, 0, st>>>(nnz, h->tperm, E.val, E.tval);
     ++h->launches;
-    k_fill<double><<<grid_for(n), 256, 0, st>>>(h->C, n, 1.0);
-    ++h->launches;
+    LP_TRY(ruiz_scale(h, o->ruiz_iters, o->ruiz_tol, E.val, E.tval, 1, nullptr, nullptr,
+                      reinterpret_cast<unsigned long long*>(h->scratch + 2 * (m + n))));
     double* rn = h->scratch;
     double* cn = h->scratch + m;
-    unsigned long long* dev = reinterpret_cast<unsigned long long*>(h->scratch + m + n);
-    for (int it = 0; it < o->ruiz_iters; ++it) {
-        k_row_inf<<<grid_for(m * 32), 256, 0, st>>>(m, h->rp, E.val, rn);
-        ++h->launches;
-        LP_CUDA_TRY(cudaMemsetAsync(cn, 0, sizeof(double) * (size_t)n, st));
-        k_col_inf<<<grid_for(nnz, 256, 8192), 256, 0, st>>>(
-            nnz, h->ci, E.val, reinterpret_cast<unsigned long long*>(cn));
-        ++h->launches;
-        LP_CUDA_TRY(cudaMemsetAsync(dev, 0, sizeof(unsigned long long), st));
-        k_ruiz_dev<<<grid_for(m + n, 256, 4096), 256, 0, st>>>(m, n, rn, cn, dev);
-        ++h->launches;
-        LP_CUDA_TRY(cudaGetLastError());
-        unsigned long long hdev = 0;
-        LP_CUDA_TRY(cudaMemcpyAsync(&hdev, dev, sizeof(hdev), cudaMemcpyDeviceToHost, st));
-        LP_CUDA_TRY(cudaStreamSynchronize(st));
-        double dv;
-        std::memcpy(&dv, &hdev, sizeof(dv));
-        if (dv <= o->ruiz_tol) break;
-        k_ruiz_factors<<<grid_for(m), 256, 0, st>>>(m, rn, h->R);
-        ++h->launches;
-        k_ruiz_factors<<<grid_for(n), 256, 0, st>>>(n, cn, h->C);
-        ++h->launches;
-        k_scale_vals<<<grid_for(nnz, 256, 8192), 256, 0, st>>>(nnz, h->krow, h->ci, rn, cn, E.val);
-        ++h->launches;
-        LP_CUDA_TRY(cudaGetLastError());
-    }
     if (o->pock_chambolle) {
         k_pc_sums<<<grid_for(m + n), 256, 0, st>>>(m, n, h->rp, h->trp, h->tperm, E.val,
                                                    o->pc_alpha, rn, cn);
@@ -729,13 +898,12 @@ lp_status setup_scale(Handle* h, const lp_opts* o, double* normK)
         ++h->launches;
         k_scale_vals<<<grid_for(nnz, 256, 8192), 256, 0, st>>>(nnz, h->krow, h->ci, rn, cn, E.val);
         ++h->launches;
+        k_gather_cast<double><<<grid_for(nnz, 256, 8192), 256, 0, st>>>(nnz, h->tperm, E.val, E.tval);
+        ++h->launches;
         LP_CUDA_TRY(cudaGetLastError());
     }
     k_scale_vectors<<<grid_for(m + n), 256, 0, st>>>(m, n, h->R, h->C, h->c0, h->q0, h->l0, h->u0,
                                                      E.c, E.q, E.l, E.u);
-    ++h->launches;
-    LP_CUDA_TRY(cudaMemsetAsync(E.tval, 0, pad8(nnz) * sizeof(double), st));
-    k_gather_cast<double><<<grid_for(nnz, 256, 8192), 256, 0, st>>>(nnz, h->tperm, E.val, E.tval);
     ++h->launches;
     LP_CUDA_TRY(cudaGetLastError());
     LP_TRY(res_values<double>(h));
