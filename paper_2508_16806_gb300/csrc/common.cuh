@@ -214,6 +214,10 @@ struct SlicedSide {
     int64_t entries = 0;
     const int4* slice = nullptr;      // first entry / 32, steps, log2 of the lanes per row, first
                                       // row of the list; the longest first
+    // a batch: place of the slice in row order; by that place its LP and a partial (twice); first
+    // place of each LP [B + 1]
+    const int32_t *tag = nullptr, *lp = nullptr, *lp0 = nullptr;
+    double* part = nullptr;
     const int32_t* row = nullptr;     // rows of the slices (-1: none)
     const int32_t* idx = nullptr;     // column of each entry (-1: padding)
     const int32_t* perm = nullptr;    // its nonzero
@@ -609,6 +613,12 @@ template <typename T> lp_status res_values(Handle* h);   // the slices' values f
 template <typename T> lp_status launch_res_period(Handle* h, cudaStream_t st, bool halpern);
 lp_status launch_res_power(Handle* h, cudaStream_t st, int iters, double* out);
 // sliced.cu: the sliced rows of an engine's sides, and their values from val, tval
+// One side; lp0: the rows at which the LPs of a batch begin [B + 1] (one LP: nullptr)
+template <typename T>
+lp_status slice_side(Handle* h, const std::vector<int64_t>& hrp, const int64_t* rp, const int32_t* ci,
+                     int64_t x_len, const std::vector<int64_t>* lp0, SlicedSide* out);
+// its values from those of the side's nonzeros
+template <typename T> lp_status slice_refresh(Handle* h, const SlicedSide& S, const T* val);
 template <typename T> lp_status slice_plan(Handle* h);
 template <typename T> lp_status slice_values(Handle* h);
 // grad.cu

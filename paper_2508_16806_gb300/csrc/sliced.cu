@@ -9,20 +9,18 @@ namespace pdhg {
 
 namespace {
 
-// The rows of one window by falling length (ties: the lower row first) and its slices,
+// The rows of one window (wst: first rows; at most W) by falling length (ties: the lower row first) and its slices,
 // one block of W threads per window.  Count only (slice = nullptr): cnt[w] =
 // (slices, steps, entries of the row list, 0).  Else the records and the row list go to
 // their places off[w] = (first slice, first step, first entry of the row list, 0).
 template <int W>
 __global__ void __launch_bounds__(W)
-k_slice_rows(int64_t rows, const int64_t* rp, int4* cnt, const int4* off, int4* slice, int32_t* list)
+k_slice_rows(const int32_t* wst, const int64_t* rp, int4* cnt, const int4* off, int4* slice, int32_t* list)
 {
     __shared__ int len[W], srt[W], who[W];
     const int t = threadIdx.x;
-    const int64_t r = (int64_t)blockIdx.x * W + t;
-    const int n = (int)(rows - (int64_t)blockIdx.x * W < W
-                            ? rows - (int64_t)blockIdx.x * W
-                            : W);
+    const int r0 = wst[blockIdx.x], n = wst[blockIdx.x + 1] - r0;
+    const int64_t r = r0 + t;
     len[t] = t < n ? (int)(rp[r + 1] - rp[r]) : -1;
     __syncthreads();
     int k = 0;
@@ -40,8 +38,7 @@ k_slice_rows(int64_t rows, const int64_t* rp, int4* cnt, const int4* off, int4* 
         if (slice) {
             slice[o.x + ns] = make_int4(o.y + steps, st, lg, o.z + nl);
             for (int j = 0; j < per; ++j)
-                list[o.z + nl + j] =
-                    i + j < n ? (int32_t)((int64_t)blockIdx.x * W + who[i + j]) : -1;
+                list[o.z + nl + j] = i + j < n ? r0 + who[i + j] : -1;
         }
         ++ns;
         steps += st;
@@ -79,9 +76,11 @@ __global__ void k_slice_values(int64_t entries, const int32_t* perm, const T* va
         out[i] = perm[i] >= 0 ? val[perm[i]] : T(0);
 }
 
+}  // namespace
+
 template <typename T>
 lp_status slice_side(Handle* h, const std::vector<int64_t>& hrp, const int64_t* rp, const int32_t* ci,
-                     int64_t x_len, int sms, SlicedSide* out)
+                     int64_t x_len, const std::vector<int64_t>* lp0, SlicedSide* out)
 {
     constexpr int W = kSliceWin<T>;
     SlicedSide S;
@@ -92,13 +91,28 @@ lp_status slice_side(Handle* h, const std::vector<int64_t>& hrp, const int64_t* 
     if (nnz == 0 || (double)nnz > 48.0 * (double)rows) return LP_OK;
     int64_t maxrow = 0;
     for (int64_t r = 0; r < rows; ++r) maxrow = std::max(maxrow, hrp[(size_t)r + 1] - hrp[(size_t)r]);
-    if (maxrow > 8192 || x_len * (int64_t)sizeof(T) <= kL1GatherBytes) return LP_OK;
+    if (maxrow > 8192 || x_len * (int64_t)sizeof(T) <= kL1GatherBytes || rows >= ((int64_t)1 << 31))
+        return LP_OK;
     cudaStream_t st = h->stream;
-    const int nwin = (int)((rows + W - 1) / W);
+    int sms = 0;
+    LP_CUDA_TRY(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, h->device));
+    // windows of W rows, none across two LPs
+    const size_t B = lp0 ? lp0->size() - 1 : 1;
+    std::vector<int32_t> wst, wfirst(B + 1);
+    for (size_t k = 0; k < B; ++k) {
+        wfirst[k] = (int32_t)wst.size();
+        const int64_t e = lp0 ? (*lp0)[k + 1] : rows;
+        for (int64_t r = lp0 ? (*lp0)[k] : 0; r < e; r += W) wst.push_back((int32_t)r);
+    }
+    const int nwin = wfirst[B] = (int32_t)wst.size();
+    wst.push_back((int32_t)rows);
     std::vector<int4> w((size_t)nwin);
     int4 *dw = nullptr, *raw = nullptr;
+    int32_t* dst = nullptr;
     LP_TRY(dev_alloc_n(h, &dw, (size_t)nwin));
-    k_slice_rows<W><<<nwin, W, 0, st>>>(rows, rp, dw, nullptr, nullptr, nullptr);
+    LP_TRY(dev_alloc_n(h, &dst, wst.size()));
+    LP_CUDA_TRY(cudaMemcpyAsync(dst, wst.data(), wst.size() * 4, cudaMemcpyHostToDevice, st));
+    k_slice_rows<W><<<nwin, W, 0, st>>>(dst, rp, dw, nullptr, nullptr, nullptr);
     LP_CUDA_TRY(cudaGetLastError());
     LP_CUDA_TRY(cudaMemcpyAsync(w.data(), dw, (size_t)nwin * sizeof(int4), cudaMemcpyDeviceToHost, st));
     LP_CUDA_TRY(cudaStreamSynchronize(st));
@@ -116,6 +130,7 @@ lp_status slice_side(Handle* h, const std::vector<int64_t>& hrp, const int64_t* 
     const size_t need = (size_t)ns * sizeof(int4) + (size_t)nl * 4 + (size_t)steps * 32 * (8 + sizeof(T));
     if (steps * 32 >= ((int64_t)1 << 31) || nl >= ((int64_t)1 << 31) || need > avail / 4) {
         dev_free(h, dw);
+        dev_free(h, dst);
         return LP_OK;
     }
     int32_t *list = nullptr, *idx = nullptr, *perm = nullptr;
@@ -126,7 +141,7 @@ lp_status slice_side(Handle* h, const std::vector<int64_t>& hrp, const int64_t* 
     LP_TRY(dev_alloc_n(h, &perm, (size_t)steps * 32));
     LP_TRY(dev_alloc_n(h, &val, (size_t)steps * 32));
     LP_CUDA_TRY(cudaMemcpyAsync(dw, w.data(), (size_t)nwin * sizeof(int4), cudaMemcpyHostToDevice, st));
-    k_slice_rows<W><<<nwin, W, 0, st>>>(rows, rp, nullptr, dw, raw, list);
+    k_slice_rows<W><<<nwin, W, 0, st>>>(dst, rp, nullptr, dw, raw, list);
     k_slice_fill<<<4 * 1216, 256, 0, st>>>((int)ns, raw, list, rp, ci, idx, perm);
     LP_CUDA_TRY(cudaGetLastError());
     h->launches += 3;
@@ -139,10 +154,35 @@ lp_status slice_side(Handle* h, const std::vector<int64_t>& hrp, const int64_t* 
     std::vector<int64_t> at((size_t)mx + 2, 0);
     for (const int4& q : rec) ++at[(size_t)(mx - q.y) + 1];
     for (int k = 0; k <= mx; ++k) at[(size_t)k + 1] += at[(size_t)k];
-    for (const int4& q : rec) ord[(size_t)at[(size_t)(mx - q.y)]++] = q;
+    std::vector<int32_t> tag((size_t)ns);
+    for (int64_t i = 0; i < ns; ++i) {
+        const int64_t p = at[(size_t)(mx - rec[(size_t)i].y)]++;
+        ord[(size_t)p] = rec[(size_t)i];
+        tag[(size_t)p] = (int32_t)i;
+    }
     LP_CUDA_TRY(cudaMemcpyAsync(raw, ord.data(), (size_t)ns * sizeof(int4), cudaMemcpyHostToDevice, st));
+    std::vector<int32_t> lp, lps(B + 1, (int32_t)ns);
+    if (lp0) {
+        lp.resize((size_t)ns);
+        for (size_t k = 0; k < B; ++k)
+            lps[k] = wfirst[k] < nwin ? w[(size_t)wfirst[k]].x : (int32_t)ns;
+        for (size_t k = 0; k < B; ++k)
+            std::fill(lp.begin() + lps[k], lp.begin() + lps[k + 1], (int32_t)k);
+        int32_t *dtag = nullptr, *dlp = nullptr, *dlp0 = nullptr;
+        LP_TRY(dev_alloc_n(h, &dtag, (size_t)ns));
+        LP_TRY(dev_alloc_n(h, &dlp, (size_t)ns));
+        LP_TRY(dev_alloc_n(h, &dlp0, B + 1));
+        LP_TRY(dev_alloc_n(h, &S.part, 2 * (size_t)ns));
+        LP_CUDA_TRY(cudaMemcpyAsync(dtag, tag.data(), (size_t)ns * 4, cudaMemcpyHostToDevice, st));
+        LP_CUDA_TRY(cudaMemcpyAsync(dlp, lp.data(), (size_t)ns * 4, cudaMemcpyHostToDevice, st));
+        LP_CUDA_TRY(cudaMemcpyAsync(dlp0, lps.data(), (B + 1) * 4, cudaMemcpyHostToDevice, st));
+        S.tag = dtag;
+        S.lp = dlp;
+        S.lp0 = dlp0;
+    }
     LP_CUDA_TRY(cudaStreamSynchronize(st));
     dev_free(h, dw);
+    dev_free(h, dst);
     S.slice = raw;
     S.row = list;
     S.idx = idx;
@@ -156,16 +196,23 @@ lp_status slice_side(Handle* h, const std::vector<int64_t>& hrp, const int64_t* 
     return LP_OK;
 }
 
-}  // namespace
-
 template <typename T>
 lp_status slice_plan(Handle* h)
 {
     Engine<T>& E = engine_of<T>(h);
-    int sms = 0;
-    LP_CUDA_TRY(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, h->device));
-    LP_TRY(slice_side<T>(h, h->h_rp, h->rp, h->ci, h->n, sms, &E.slK));
-    LP_TRY(slice_side<T>(h, h->h_trp, h->trp, h->tci, h->m, sms, &E.slT));
+    LP_TRY(slice_side<T>(h, h->h_rp, h->rp, h->ci, h->n, nullptr, &E.slK));
+    LP_TRY(slice_side<T>(h, h->h_trp, h->trp, h->tci, h->m, nullptr, &E.slT));
+    return LP_OK;
+}
+
+template <typename T>
+lp_status slice_refresh(Handle* h, const SlicedSide& S, const T* val)
+{
+    if (!S.on) return LP_OK;
+    const int64_t g = std::min<int64_t>(4 * 1216, (S.entries + 255) / 256);
+    k_slice_values<T><<<(int)g, 256, 0, h->stream>>>(S.entries, S.perm, val, static_cast<T*>(S.val));
+    ++h->launches;
+    LP_CUDA_TRY(cudaGetLastError());
     return LP_OK;
 }
 
@@ -173,21 +220,19 @@ template <typename T>
 lp_status slice_values(Handle* h)
 {
     Engine<T>& E = engine_of<T>(h);
-    for (int side = 0; side < 2; ++side) {
-        const SlicedSide& S = side ? E.slT : E.slK;
-        if (!S.on) continue;
-        const int64_t g = std::min<int64_t>(4 * 1216, (S.entries + 255) / 256);
-        k_slice_values<T><<<(int)g, 256, 0, h->stream>>>(S.entries, S.perm, side ? E.tval : E.val,
-                                                         static_cast<T*>(S.val));
-        ++h->launches;
-    }
-    LP_CUDA_TRY(cudaGetLastError());
-    return LP_OK;
+    LP_TRY(slice_refresh<T>(h, E.slK, E.val));
+    return slice_refresh<T>(h, E.slT, E.tval);
 }
 
 template lp_status slice_plan<double>(Handle*);
 template lp_status slice_plan<float>(Handle*);
 template lp_status slice_values<double>(Handle*);
 template lp_status slice_values<float>(Handle*);
+template lp_status slice_side<double>(Handle*, const std::vector<int64_t>&, const int64_t*, const int32_t*,
+                                      int64_t, const std::vector<int64_t>*, SlicedSide*);
+template lp_status slice_side<float>(Handle*, const std::vector<int64_t>&, const int64_t*, const int32_t*,
+                                     int64_t, const std::vector<int64_t>*, SlicedSide*);
+template lp_status slice_refresh<double>(Handle*, const SlicedSide&, const double*);
+template lp_status slice_refresh<float>(Handle*, const SlicedSide&, const float*);
 
 }  // namespace pdhg

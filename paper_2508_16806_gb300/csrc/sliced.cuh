@@ -69,6 +69,34 @@ __device__ __forceinline__ void slice_steps(const int32_t* __restrict__ si, cons
     for (int u = 0; u < U; ++u) a = fma(v[u], xv[u], a);
 }
 
+// One slice: the rows' sums and, on each row's owner lane, their epilogue.
+template <typename T, class Epi>
+__device__ __forceinline__ void slice_run(const SlicedSide& S, const T* __restrict__ val, const int4 d,
+                                          const T* __restrict__ x, Epi& epi, typename Epi::Acc& acc)
+{
+    const int lane = threadIdx.x & 31;
+    const int row = __ldg(S.row + d.w + (lane >> d.z));
+    const bool own = row >= 0 && (lane & ((1 << d.z) - 1)) == 0;
+    const int32_t* __restrict__ si = S.idx + (size_t)d.x * 32 + lane;
+    const T* __restrict__ sv = val + (size_t)d.x * 32 + lane;
+    typename Epi::Pre pre;
+    if (own) pre = epi.load(row);
+    T a = T(0);
+    int n = d.y;
+    for (; n >= 8; n -= 8, si += 256, sv += 256) slice_steps<8, T>(si, sv, x, a);
+    if (n >= 4) {
+        slice_steps<4, T>(si, sv, x, a);
+        n -= 4, si += 128, sv += 128;
+    }
+    if (n >= 2) {
+        slice_steps<2, T>(si, sv, x, a);
+        n -= 2, si += 64, sv += 64;
+    }
+    if (n >= 1) slice_steps<1, T>(si, sv, x, a);
+    for (int o = (1 << d.z) >> 1; o > 0; o >>= 1) a += __shfl_xor_sync(0xffffffffu, a, o);
+    if (own) epi.row(row, a, pre, acc);
+}
+
 template <typename T, class Epi>
 __global__ void __launch_bounds__(kSpmvNT, kSliceBlocks<T>)
 k_sliced(const SlicedSide S, const T* __restrict__ val, Epi epi)
@@ -76,7 +104,6 @@ k_sliced(const SlicedSide S, const T* __restrict__ val, Epi epi)
     if (!epi.begin()) return;
     const T* __restrict__ x = epi.xin();
     typename Epi::Acc acc;
-    const int lane = threadIdx.x & 31;
     const int nw = gridDim.x * (kSpmvNT / 32), s1 = S.nslice;
     int s = (threadIdx.x >> 5) * gridDim.x + blockIdx.x;
     // first entry / 32, steps, log2 of the lanes per row, first row of the list
@@ -86,29 +113,43 @@ k_sliced(const SlicedSide S, const T* __restrict__ val, Epi epi)
         s += nw;
         int4 dn = d;
         if (s < s1) dn = __ldg(S.slice + s);
-        const int row = __ldg(S.row + d.w + (lane >> d.z));
-        const bool own = row >= 0 && (lane & ((1 << d.z) - 1)) == 0;
-        const int32_t* __restrict__ si = S.idx + (size_t)d.x * 32 + lane;
-        const T* __restrict__ sv = val + (size_t)d.x * 32 + lane;
-        typename Epi::Pre pre;
-        if (own) pre = epi.load(row);
-        T a = T(0);
-        int n = d.y;
-        for (; n >= 8; n -= 8, si += 256, sv += 256) slice_steps<8, T>(si, sv, x, a);
-        if (n >= 4) {
-            slice_steps<4, T>(si, sv, x, a);
-            n -= 4, si += 128, sv += 128;
-        }
-        if (n >= 2) {
-            slice_steps<2, T>(si, sv, x, a);
-            n -= 2, si += 64, sv += 64;
-        }
-        if (n >= 1) slice_steps<1, T>(si, sv, x, a);
-        for (int o = (1 << d.z) >> 1; o > 0; o >>= 1) a += __shfl_xor_sync(0xffffffffu, a, o);
-        if (own) epi.row(row, a, pre, acc);
+        slice_run<T, Epi>(S, val, d, x, epi, acc);
         d = dn;
     }
     epi.finish(acc);
+}
+
+// The same for a batch: a slice lies within one LP, whose state the epilogue takes
+// (and whose finish skips it); its partials go to the slice's place in row order.
+template <typename T, class Epi>
+__global__ void __launch_bounds__(kSpmvNT, kSliceBlocks<T>)
+k_sliced_lp(const SlicedSide S, const T* __restrict__ val, Epi epi)
+{
+    typename Epi::Acc acc;
+    const int nw = gridDim.x * (kSpmvNT / 32), s1 = S.nslice;
+    int s = (threadIdx.x >> 5) * gridDim.x + blockIdx.x;
+    int4 d = make_int4(0, 0, 0, 0);
+    int t = 0;
+    if (s < s1) {
+        d = __ldg(S.slice + s);
+        t = __ldg(S.tag + s);
+    }
+    while (s < s1) {
+        s += nw;
+        int4 dn = d;
+        int tn = t;
+        if (s < s1) {
+            dn = __ldg(S.slice + s);
+            tn = __ldg(S.tag + s);
+        }
+        if (epi.live(t)) {
+            epi.task_start(t);
+            slice_run<T, Epi>(S, val, d, epi.xin(), epi, acc);
+            epi.task_done(t, acc);
+        }
+        d = dn;
+        t = tn;
+    }
 }
 
 // K x (side_t = false) or K^T y with an epilogue: sliced rows where the engine has
