@@ -57,3 +57,21 @@ def test_sliced_products(L, m, n):
     b = prob.solve(tol=1e-14, max_iters=20)
     assert np.array_equal(a[0], b[0]) and np.array_equal(a[1], b[1])
     prob.close()
+
+
+@pytest.mark.parametrize("rows", [[2, 31, 255, 256, 257, 9000, 20011], [30000, 1, 30001]])
+def test_sliced_batch_tracks_single_solves(L, rows):
+    """Slices of several LPs side by side (windows cut at LP ends): 64 fixed steps of each LP
+    are those of its own solve, to the bound of the batch's other tests (1e-10)."""
+    rng = np.random.default_rng(len(rows))
+    lps = [synth.random_planted(m, 2 * m, lengths=rng.integers(1, min(2 * m, 21) + 1, m), seed=m)
+           for m in rows]
+    batch = L.Batch(lps)
+    out = batch.solve(tol=1e-13, max_iters=64, adaptive_step=0)
+    for lp, (x, y, info) in zip(lps, out):
+        prob = L.Problem(lp)
+        xs, ys, si, _ = prob.solve(tol=1e-13, max_iters=64, adaptive_step=0)
+        assert info["status"] == si["status"] and info["iters"] == si["iters"]
+        assert rel(x, xs) <= 1e-10 and rel(y, ys) <= 1e-10
+        prob.close()
+    batch.close()
