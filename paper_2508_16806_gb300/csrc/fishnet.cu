@@ -27,14 +27,15 @@ namespace {
 constexpr int kFW = 8;             // warps per block of the block-SpMM kernels
 constexpr int kFGrid = 152 * 16;   // grid cap of the block-SpMM kernels (persistent rows loop)
 
-// out[r, p] = sum_k val_k X[col_k, p] for the rows r of a CSR matrix; X is row
-// major with P columns (a power of two, 1..64).  One warp per row: lane l serves
-// column l % P (and l + 32 when P = 64); for P < 32 the 32 / P lane groups take
-// every (32 / P)-th nonzero of each batch of 32 and are added by a fixed
-// butterfly.  Each gathered row of X is P contiguous values (coalesced).
 // Rows with more nonzeros than this go to k_spmm_long (a block per row), so that
-// no single warp walks a power-law row of thousands of nonzeros alone.
-constexpr int64_t kLongRow = 32 * kFW;
+// no lane walks a power-law row of thousands of nonzeros alone.
+constexpr int64_t kLongRow = 128;
+
+// V consecutive columns of a point block's row
+template <typename T, int V>
+struct alignas(sizeof(T) * V) Vec {
+    T v[V];
+};
 
 // Accumulates the batches b0, b0 + stride, ... (32 nonzeros each) of row [s, e)
 // into a0 (and a1 for P = 64); every lane of the warp calls it.
@@ -63,28 +64,46 @@ __device__ __forceinline__ void spmm_row_part(const int32_t* __restrict__ ci,
     }
 }
 
-template <typename T, class Epi>
+// out[r, p] = sum_k val_k X[col_k, p] for the rows r of a CSR matrix; X is row major with
+// P columns (a power of two, 1..64).  P / V lanes take a row, V columns (16 bytes where
+// P allows) each, and walk its nonzeros in order, eight gathers in flight (past the end:
+// the last entry again, times zero).  What bounds it is the chain start -> column -> gather
+// -> epilogue and, for many columns, the L2 bytes of the gathers; so many rows at once and
+// few instructions each.  50,000 x 100,000 LP, 625,000 nonzeros, P from 32 to 2, averages: a
+// warp per row 34 us (K^T side) and 24 us (K side); so 12.6 us and 13.0 us,
+// a call 11.4 -> 7.9 ms.
+template <typename T, int V, class Epi>
 __global__ void __launch_bounds__(kFW * 32)
 k_spmm(const int64_t* __restrict__ rp, const int32_t* __restrict__ ci,
        const T* __restrict__ val, int64_t rows, int P, const T* __restrict__ X, Epi epi)
 {
-    const unsigned full = 0xffffffffu;
-    const int lane = threadIdx.x & 31;
-    const int Pl = P < 32 ? P : 32;
-    const int G = 32 / Pl;
-    const int g = lane / Pl, p = lane % Pl;
-    const bool two = P == 64;
-    for (int64_t r = (int64_t)blockIdx.x * kFW + (threadIdx.x >> 5); r < rows;
-         r += (int64_t)gridDim.x * kFW) {
+    using W = Vec<T, V>;
+    const int lr = P / V, per = kFW * 32 / lr;
+    const int p = (int)(threadIdx.x & (lr - 1)) * V;
+    for (int64_t r = (int64_t)blockIdx.x * per + threadIdx.x / lr; r < rows;
+         r += (int64_t)gridDim.x * per) {
         const int64_t s = rp[r], e = rp[r + 1];
         if (e - s > kLongRow) continue;
-        T a0 = 0, a1 = 0;
-        spmm_row_part(ci, val, s, e, 32, P, X, lane, G, g, p, two, a0, a1);
-        for (int o = Pl; o < 32; o <<= 1) a0 += __shfl_xor_sync(full, a0, o);
-        if (g == 0) {
-            epi.row(r, p, a0);
-            if (two) epi.row(r, p + 32, a1);
+        const auto pre = epi.template load<V>(r, p);
+        W a;
+#pragma unroll
+        for (int i = 0; i < V; ++i) a.v[i] = T(0);
+        for (int64_t k = s; k < e; k += 8) {
+            int c[8];
+            T v[8];
+            W x[8];
+#pragma unroll
+            for (int u = 0; u < 8; ++u) c[u] = ci[k + u < e ? k + u : e - 1];
+#pragma unroll
+            for (int u = 0; u < 8; ++u) v[u] = val[k + u < e ? k + u : e - 1];
+#pragma unroll
+            for (int u = 0; u < 8; ++u) x[u] = *reinterpret_cast<const W*>(X + (int64_t)c[u] * P + p);
+#pragma unroll
+            for (int u = 0; u < 8; ++u)
+#pragma unroll
+                for (int i = 0; i < V; ++i) a.v[i] = fma(k + u < e ? v[u] : T(0), x[u].v[i], a.v[i]);
         }
+        epi.template row<V>(r, p, a, pre);
     }
 }
 
@@ -122,18 +141,24 @@ k_spmm_long(const int64_t* __restrict__ rp, const int32_t* __restrict__ ci,
                 t0 += sh[w][p];
                 if (two) t1 += sh[w][p + 32];
             }
-            epi.row(r, p, t0);
-            if (two) epi.row(r, p + 32, t1);
+            epi.template row<1>(r, p, Vec<T, 1>{{t0}}, epi.template load<1>(r, p));
+            if (two) epi.template row<1>(r, p + 32, Vec<T, 1>{{t1}}, epi.template load<1>(r, p + 32));
         }
         __syncthreads();
     }
 }
 
+// Epilogues: load<V> fetches the row's operands ahead of the sums, row<V> takes the sums
+// of columns p .. p + V - 1.
 template <typename T>
 struct FStore {
     T* out;
     int P;
-    __device__ void row(int64_t r, int p, T v) const { out[r * P + p] = v; }
+    template <int V> __device__ int load(int64_t, int) const { return 0; }
+    template <int V> __device__ void row(int64_t r, int p, const Vec<T, V>& s, int) const
+    {
+        *reinterpret_cast<Vec<T, V>*>(out + r * P + p) = s;
+    }
 };
 
 // x' = proj_X(x - tau (c - K^T y)) per column (Algorithm 1, theta = 1)
@@ -144,13 +169,22 @@ struct FPrimal {
     const T *c, *l, *u;
     T tau;
     int P;
-    __device__ void row(int64_t j, int p, T kty) const
+    template <int V> struct Pre { Vec<T, V> x; T c, l, u; };
+    template <int V> __device__ Pre<V> load(int64_t j, int p) const
     {
-        const int64_t t = j * P + p;
-        T v = X[t] - tau * (c[j] - kty);
-        if (v < l[j]) v = l[j];
-        if (v > u[j]) v = u[j];
-        Xn[t] = v;
+        return {*reinterpret_cast<const Vec<T, V>*>(X + j * P + p), c[j], l[j], u[j]};
+    }
+    template <int V> __device__ void row(int64_t j, int p, const Vec<T, V>& s, const Pre<V>& o) const
+    {
+        Vec<T, V> w;
+#pragma unroll
+        for (int i = 0; i < V; ++i) {
+            T v = o.x.v[i] - tau * (o.c - s.v[i]);
+            if (v < o.l) v = o.l;
+            if (v > o.u) v = o.u;
+            w.v[i] = v;
+        }
+        *reinterpret_cast<Vec<T, V>*>(Xn + j * P + p) = w;
     }
 };
 
@@ -164,13 +198,23 @@ struct FDual {
     const uint8_t* sense;
     T sigma;
     int P;
-    __device__ void row(int64_t i, int p, T kxn) const
+    template <int V> struct Pre { Vec<T, V> y, kx; T q; bool ge; };
+    template <int V> __device__ Pre<V> load(int64_t i, int p) const
     {
-        const int64_t t = i * P + p;
-        T v = Y[t] + sigma * (q[i] - (T(2) * kxn - KX[t]));
-        if (sense[i] && v < T(0)) v = T(0);
-        Yn[t] = v;
-        KX[t] = kxn;
+        return {*reinterpret_cast<const Vec<T, V>*>(Y + i * P + p),
+                *reinterpret_cast<const Vec<T, V>*>(KX + i * P + p), q[i], sense[i] != 0};
+    }
+    template <int V> __device__ void row(int64_t i, int p, const Vec<T, V>& s, const Pre<V>& o) const
+    {
+        Vec<T, V> w;
+#pragma unroll
+        for (int k = 0; k < V; ++k) {
+            T v = o.y.v[k] + sigma * (o.q - (T(2) * s.v[k] - o.kx.v[k]));
+            if (o.ge && v < T(0)) v = T(0);
+            w.v[k] = v;
+        }
+        *reinterpret_cast<Vec<T, V>*>(Yn + i * P + p) = w;
+        *reinterpret_cast<Vec<T, V>*>(KX + i * P + p) = s;
     }
 };
 
@@ -292,14 +336,6 @@ int ew_blocks(int64_t count)
     return (int)g;
 }
 
-int spmm_blocks(int64_t rows)
-{
-    int64_t g = (rows + kFW - 1) / kFW;
-    if (g < 1) g = 1;
-    if (g > kFGrid) g = kFGrid;
-    return (int)g;
-}
-
 // Rows of a CSR orientation with more than kLongRow nonzeros (host).
 std::vector<int32_t> long_rows(const std::vector<int64_t>& rp)
 {
@@ -309,12 +345,21 @@ std::vector<int32_t> long_rows(const std::vector<int64_t>& rp)
     return out;
 }
 
-// One block product: the short rows (a warp each), then the long ones (a block each).
+// One block product: the short rows, then the long ones (a block each).
 template <typename T, class Epi>
 void spmm(Handle* h, const int64_t* rp, const int32_t* ci, const T* val, int64_t rows, int P,
           const T* X, const int32_t* lrows, int nlong, const Epi& epi)
 {
-    k_spmm<T, Epi><<<spmm_blocks(rows), kFW * 32, 0, h->stream>>>(rp, ci, val, rows, P, X, epi);
+    constexpr int W = 16 / sizeof(T);   // columns of a 16-byte load
+    const int V = P < W ? P : W;
+    const int64_t per = kFW * 32 / (P / V);
+    const int grid = (int)std::max<int64_t>(1, std::min<int64_t>((rows + per - 1) / per, kFGrid));
+    if (V == 4)
+        k_spmm<T, W, Epi><<<grid, kFW * 32, 0, h->stream>>>(rp, ci, val, rows, P, X, epi);
+    else if (V == 2)
+        k_spmm<T, 2, Epi><<<grid, kFW * 32, 0, h->stream>>>(rp, ci, val, rows, P, X, epi);
+    else
+        k_spmm<T, 1, Epi><<<grid, kFW * 32, 0, h->stream>>>(rp, ci, val, rows, P, X, epi);
     ++h->launches;
     if (nlong > 0) {
         k_spmm_long<T, Epi><<<std::min(nlong, kFGrid), kFW * 32, 0, h->stream>>>(
