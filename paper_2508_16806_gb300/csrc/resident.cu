@@ -707,25 +707,31 @@ const void* res_kernel(int what, bool sm)
 }
 
 // Launch of a resident kernel: a cooperative grid, or one cluster.
-lp_status res_launch(const ResPlan& R, cudaStream_t st, const void* f, void** args)
+cudaLaunchConfig_t res_config(const ResPlan& R, cudaStream_t st, cudaLaunchAttribute* at)
 {
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((unsigned)R.ncta);
     cfg.blockDim = dim3((unsigned)R.threads);
     cfg.dynamicSmemBytes = R.smem;
     cfg.stream = st;
-    cudaLaunchAttribute at[1];
     if (R.cluster) {
-        at[0].id = cudaLaunchAttributeClusterDimension;
-        at[0].val.clusterDim.x = (unsigned)R.ncta;
-        at[0].val.clusterDim.y = 1;
-        at[0].val.clusterDim.z = 1;
+        at->id = cudaLaunchAttributeClusterDimension;
+        at->val.clusterDim.x = (unsigned)R.ncta;
+        at->val.clusterDim.y = 1;
+        at->val.clusterDim.z = 1;
     } else {
-        at[0].id = cudaLaunchAttributeCooperative;
-        at[0].val.cooperative = 1;
+        at->id = cudaLaunchAttributeCooperative;
+        at->val.cooperative = 1;
     }
     cfg.attrs = at;
     cfg.numAttrs = 1;
+    return cfg;
+}
+
+lp_status res_launch(const ResPlan& R, cudaStream_t st, const void* f, void** args)
+{
+    cudaLaunchAttribute at;
+    const cudaLaunchConfig_t cfg = res_config(R, st, &at);
     LP_CUDA_TRY(cudaLaunchKernelExC(&cfg, f, args));
     return LP_OK;
 }
@@ -785,6 +791,15 @@ lp_status res_plan(Handle* h)
         LP_CUDA_TRY(cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dyn));
         if (R.cluster) {
             LP_CUDA_TRY(cudaFuncSetAttribute(f, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
+            // a device (or a part of one) without room for such a cluster keeps the launches
+            // per product
+            int fit = 0;
+            cudaLaunchAttribute at;
+            const cudaLaunchConfig_t cfg = res_config(R, h->stream, &at);
+            if (cudaOccupancyMaxActiveClusters(&fit, f, &cfg) != cudaSuccess || fit < 1) {
+                (void)cudaGetLastError();
+                return LP_OK;
+            }
         } else {
             int occ = 0;
             LP_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, f, R.threads, R.smem));
