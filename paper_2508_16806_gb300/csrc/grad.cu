@@ -18,6 +18,7 @@
 #include <type_traits>
 
 #include "common.cuh"
+#include "control.cuh"
 #include "sliced.cuh"
 
 namespace pdhg {
@@ -32,21 +33,34 @@ inline int ew_grid_g(int64_t count)
     return (int)g;
 }
 
-// x' = clamp(x - tau (c - K^T y), l, u); mask of the strict interior
+// What bounds an unrolled step of a mid-size LP is its chain of short launches and, in the
+// derivative of the nonzeros, gathers and FP64 instructions.  The elementwise parts
+// therefore ride on the products' epilogues (two launches a forward step, two a reverse
+// step), and the derivative of the nonzeros is taken kGSteps reverse steps at a time
+// (k_g_pack, k_g_sddmm).
+
+// K^T y + primal step: x' = clamp(x - tau (c - K^T y), l, u); mask of the strict interior
 template <typename T>
-__global__ void k_g_primal(const T* x, const T* kty, const T* c, const T* l, const T* u,
-                           const double* coef, T* xn, uint8_t* mx, int64_t n)
-{
-    const T tau = (T)coef[0];
-    for (int64_t j = (int64_t)blockIdx.x * kEW + threadIdx.x; j < n; j += (int64_t)gridDim.x * kEW) {
-        const T v = x[j] - tau * (c[j] - kty[j]);
-        T o = v;
-        if (o < l[j]) o = l[j];
-        if (o > u[j]) o = u[j];
-        xn[j] = o;
-        if (mx) mx[j] = (l[j] < v && v < u[j]) ? 1 : 0;
+struct EpiGPrimal {
+    PDHG_SINGLE_LP_TASK_HOOKS
+    const T* y;          // being multiplied
+    const T* x;
+    const T *c, *l, *u;
+    const double* coef;  // [0] = tau
+    T* xn;
+    uint8_t* mx;
+    struct Pre { T x = 0, c = 0, l = 0, u = 0; };
+    struct Acc {};
+    __device__ bool begin() const { return true; }
+    __device__ const T* xin() const { return y; }
+    __device__ Pre load(int j) const { return Pre{x[j], c[j], l[j], u[j]}; }
+    __device__ void row(int j, T k, const Pre& p, Acc&) const {
+        const T v = p.x - (T)coef[0] * (p.c - k);
+        xn[j] = res_clamp(v, p.l, p.u);
+        if (mx) mx[j] = res_inside(v, p.l, p.u) ? 1 : 0;
     }
-}
+    __device__ void finish(Acc&) const {}
+};
 
 // K x' + dual step of the unrolled forward, with the dual mask
 template <typename T>
@@ -69,16 +83,14 @@ struct EpiGDual {
     __device__ void row(int i, T v, const Pre& p, Acc&) const {
         const T sigma = (T)coef[1];
         const T w = p.y + sigma * (p.q - (T(2) * v - p.kx));
-        T o = w;
-        if (p.ge && o < T(0)) o = T(0);
-        yn[i] = o;
+        yn[i] = p.ge ? res_pos(w) : w;
         kxn[i] = v;
-        if (my) my[i] = (!p.ge || w > T(0)) ? 1 : 0;
+        if (my) my[i] = (!p.ge || res_positive(w)) ? 1 : 0;
     }
     __device__ void finish(Acc&) const {}
 };
 
-// reverse: gv_y = M_y gy; dq += sigma gv_y
+// reverse, last step of a segment: gv_y = M_y gy; dq += sigma gv_y
 template <typename T>
 __global__ void k_g_gvy(const uint8_t* my, const T* gy, const double* coef, T* gvy, double* dq,
                         int64_t m)
@@ -91,50 +103,116 @@ __global__ void k_g_gvy(const uint8_t* my, const T* gy, const double* coef, T* g
     }
 }
 
-// reverse: gv_x = M_x (gx + 2 gxbar); dc += -tau gv_x; gx <- gv_x - gxbar
+// reverse: gxbar = -sigma K^T gv_y; gv_x = M_x (gx + 2 gxbar); dc += -tau gv_x;
+// gx <- gv_x - gxbar (epilogue of the K^T gv_y product)
 template <typename T>
-__global__ void k_g_gvx(const uint8_t* mx, T* gx, const T* gxbar, const double* coef, T* gvx,
-                        double* dc, int64_t n)
-{
-    const double tau = coef[0];
-    for (int64_t j = (int64_t)blockIdx.x * kEW + threadIdx.x; j < n; j += (int64_t)gridDim.x * kEW) {
-        const T gb = gxbar[j];
-        const T g = mx[j] ? gx[j] + T(2) * gb : T(0);
+struct EpiGvx {
+    PDHG_SINGLE_LP_TASK_HOOKS
+    const T* gvy;        // being multiplied
+    const uint8_t* mx;
+    const double* coef;  // [0] = tau, [2] = -sigma
+    T* gx;
+    T* gvx;
+    double* dc;
+    struct Pre { T gx = 0; uint8_t in = 0; };
+    struct Acc {};
+    __device__ bool begin() const { return true; }
+    __device__ const T* xin() const { return gvy; }
+    __device__ Pre load(int j) const { return Pre{gx[j], mx[j]}; }
+    __device__ void row(int j, T v, const Pre& p, Acc&) const {
+        const T gb = (T)__dmul_rn((double)v, coef[2]);   // one value in both places below
+        const T g = p.in ? p.gx + T(2) * gb : T(0);
         gvx[j] = g;
-        dc[j] += -tau * (double)g;
+        dc[j] += -coef[0] * (double)g;
         gx[j] = g - gb;
     }
-}
+    __device__ void finish(Acc&) const {}
+};
 
-// reverse: gy <- gv_y + tau K gv_x (epilogue of the K gv_x product)
+// reverse: gy = gv_y + tau K gv_x (epilogue of the K gv_x product) and, unless the segment
+// ends, the first half of the step before: gv_y = M_y gy; dq += sigma gv_y
 template <typename T>
 struct EpiGy {
     PDHG_SINGLE_LP_TASK_HOOKS
     const T* gvx;        // being multiplied
     const T* gvy;
-    const double* coef;  // [0] = tau
-    T* gy;
-    struct Pre { T g = 0; };
+    const double* coef;  // [0] = tau, [1] = sigma
+    T* gy;               // kept where the segment ends (my = nullptr)
+    const uint8_t* my;   // of the step before
+    T* gvyn;
+    double* dq;
+    struct Pre { T g = 0; uint8_t in = 0; };
     struct Acc {};
     __device__ bool begin() const { return true; }
     __device__ const T* xin() const { return gvx; }
-    __device__ Pre load(int i) const { return Pre{gvy[i]}; }
-    __device__ void row(int i, T v, const Pre& p, Acc&) const { gy[i] = p.g + (T)coef[0] * v; }
+    __device__ Pre load(int i) const { return Pre{gvy[i], my ? my[i] : (uint8_t)0}; }
+    __device__ void row(int i, T v, const Pre& p, Acc&) const {
+        const T g = p.g + (T)coef[0] * v;
+        if (!my) {
+            gy[i] = g;
+            return;
+        }
+        const T w = p.in ? g : T(0);
+        gvyn[i] = w;
+        dq[i] += coef[1] * (double)w;
+    }
     __device__ void finish(Acc&) const {}
 };
 
-// reverse: dA_p += -sigma gv_y_i xbar_j + tau y_i gv_x_j for every nonzero p = (i, j)
+// Reverse steps whose derivative of the nonzeros is taken together, at most.
+constexpr int kGSteps = 8;
+
+// The factors of cnt reverse steps (t, t - 1, ...) side by side, for k_g_sddmm:
+// P[j][k] = (xbar_j, gv_x_j), Q[i][k] = (-sigma gv_y_i, tau y_i).  X, Y: the iterates of
+// step t (X + n: those of t + 1); gvx, gvy: a vector per step.
 template <typename T>
-__global__ void k_g_sddmm(const int32_t* krow, const int32_t* ci, const T* gvy, const T* gvx,
-                          const T* x, const T* xn, const T* y, const double* coef, double* dvals,
-                          int64_t nnz)
+__global__ void k_g_pack(int cnt, int stride, const T* X, const T* Y, const T* gvx, const T* gvy,
+                         const double* coef, double2* P, double2* Q, int64_t n, int64_t m)
 {
     const double tau = coef[0], sigma = coef[1];
+    for (int64_t r = (int64_t)blockIdx.x * kEW + threadIdx.x; r < n + m;
+         r += (int64_t)gridDim.x * kEW) {
+        if (r < n) {
+            double xn = (double)X[n + r];
+            for (int k = 0; k < cnt; ++k) {
+                const double x = (double)X[r - k * n];
+                P[r * stride + k] = make_double2(2.0 * xn - x, (double)gvx[k * n + r]);
+                xn = x;
+            }
+        } else {
+            const int64_t i = r - n;
+            for (int k = 0; k < cnt; ++k)
+                Q[i * stride + k] = make_double2(-sigma * (double)gvy[k * m + i],
+                                                 tau * (double)Y[i - k * m]);
+        }
+    }
+}
+
+// reverse: dA_p += -sigma gv_y_i xbar_j + tau y_i gv_x_j for every nonzero p = (i, j),
+// the packed steps one after the other.  A step by itself took five gathers of a 32-byte
+// sector, 32 bytes of indices and sums, and seven FP64 instructions a nonzero; eight packed
+// steps gather two 128-byte lines and take three instructions a step.  (Two, with the
+// steps' terms added up before they meet dA, lost a third of the last digits.)
+__global__ void k_g_sddmm(const int32_t* krow, const int32_t* ci, const double2* P, const double2* Q,
+                          int cnt, int stride, double* dvals, int64_t nnz)
+{
     for (int64_t p = (int64_t)blockIdx.x * kEW + threadIdx.x; p < nnz;
          p += (int64_t)gridDim.x * kEW) {
-        const int32_t i = krow[p], j = ci[p];
-        const double xbar = 2.0 * (double)xn[j] - (double)x[j];
-        dvals[p] += -sigma * (double)gvy[i] * xbar + tau * (double)y[i] * (double)gvx[j];
+        const double2* q = Q + (int64_t)krow[p] * stride;
+        const double2* c = P + (int64_t)ci[p] * stride;
+        double t = dvals[p];
+        if (cnt == kGSteps) {
+            double2 a[kGSteps], b[kGSteps];
+#pragma unroll
+            for (int k = 0; k < kGSteps; ++k) b[k] = c[k];
+#pragma unroll
+            for (int k = 0; k < kGSteps; ++k) a[k] = q[k];
+#pragma unroll
+            for (int k = 0; k < kGSteps; ++k) t += fma(a[k].x, b[k].x, a[k].y * b[k].y);
+        } else {
+            for (int k = 0; k < cnt; ++k) t += fma(q[k].x, c[k].x, q[k].y * c[k].y);
+        }
+        dvals[p] = t;
     }
 }
 
@@ -210,35 +288,33 @@ lp_status grad_prepare(Handle* h, const lp_opts* o, double* tau, double* sigma)
     if (o->omega0 > 0.0) omega = o->omega0;
     *tau = eta / omega;
     *sigma = eta * omega;
+    LP_CUDA_TRY((spmv_prepare<T, EpiGPrimal<T>>()));
     LP_CUDA_TRY((spmv_prepare<T, EpiGDual<T>>()));
     LP_CUDA_TRY((spmv_prepare<T, EpiStore<T>>()));
+    LP_CUDA_TRY((spmv_prepare<T, EpiGvx<T>>()));
     LP_CUDA_TRY((spmv_prepare<T, EpiGy<T>>()));
     return LP_OK;
 }
 
-// One forward step from (x, y, kx, kty) into (xn, yn, kxn, ktyn), with masks.
+// One forward step from (x, y, kx) into (xn, yn, kxn), with masks.
 template <typename T>
 void forward_step(Handle* h, Engine<T>& E, const double* coef, const T* x, const T* y, const T* kx,
-                  const T* kty, T* xn, T* yn, T* kxn, T* ktyn, uint8_t* mx, uint8_t* my)
+                  T* xn, T* yn, T* kxn, uint8_t* mx, uint8_t* my)
 {
-    cudaStream_t st = h->stream;
-    k_g_primal<T><<<ew_grid_g(h->n), kEW, 0, st>>>(x, kty, E.c, E.l, E.u, coef, xn, mx, h->n);
+    EpiGPrimal<T> ep{y, x, E.c, E.l, E.u, coef, xn, mx};
+    launch_product<T>(h, E, true, h->stream, ep);
     EpiGDual<T> ed{xn, y, kx, E.q, h->sense, coef, yn, kxn, my};
-    launch_product<T>(h, E, false, st, ed);
-    EpiStore<T> et{yn, ktyn, nullptr, nullptr, nullptr};
-    launch_product<T>(h, E, true, st, et);
-    h->launches += 3;
+    launch_product<T>(h, E, false, h->stream, ed);
+    h->launches += 2;
 }
 
+// K x
 template <typename T>
-lp_status products(Handle* h, Engine<T>& E, const T* x, const T* y, T* kx, T* kty)
+lp_status product(Handle* h, Engine<T>& E, const T* x, T* kx)
 {
-    cudaStream_t st = h->stream;
     EpiStore<T> e1{x, kx, nullptr, nullptr, nullptr};
-    launch_product<T>(h, E, false, st, e1);
-    EpiStore<T> e2{y, kty, nullptr, nullptr, nullptr};
-    launch_product<T>(h, E, true, st, e2);
-    h->launches += 2;
+    launch_product<T>(h, E, false, h->stream, e1);
+    ++h->launches;
     LP_CUDA_TRY(cudaGetLastError());
     return LP_OK;
 }
@@ -282,7 +358,7 @@ lp_status grad_impl(Handle* h, const lp_opts* o, int K, int ckpt, const double* 
     T* y = E.Y[0];
     k_g_init<T><<<ew_grid_g(n + m), kEW, 0, st>>>(E.l, E.u, x, y, n, m);
     ++h->launches;
-    LP_TRY(products<T>(h, E, x, y, E.KX[0], E.KTY[0]));
+    LP_TRY(product<T>(h, E, x, E.KX[0]));
     int cur = 0;
     for (int t = 0; t < K; ++t) {
         if (backward && t % ckpt == 0) {
@@ -292,8 +368,8 @@ lp_status grad_impl(Handle* h, const lp_opts* o, int K, int ckpt, const double* 
             LP_CUDA_TRY(cudaMemcpyAsync(CY + (size_t)c * m, E.Y[cur], sizeof(T) * m,
                                         cudaMemcpyDeviceToDevice, st));
         }
-        forward_step<T>(h, E, coef, E.X[cur], E.Y[cur], E.KX[cur], E.KTY[cur], E.X[cur ^ 1],
-                        E.Y[cur ^ 1], E.KX[cur ^ 1], E.KTY[cur ^ 1], nullptr, nullptr);
+        forward_step<T>(h, E, coef, E.X[cur], E.Y[cur], E.KX[cur], E.X[cur ^ 1], E.Y[cur ^ 1],
+                        E.KX[cur ^ 1], nullptr, nullptr);
         cur ^= 1;
     }
     LP_CUDA_TRY(cudaGetLastError());
@@ -317,8 +393,9 @@ lp_status grad_impl(Handle* h, const lp_opts* o, int K, int ckpt, const double* 
     }
 
     // reverse pass
-    T *RX = nullptr, *RY = nullptr, *gx = nullptr, *gy = nullptr, *gvx = nullptr, *gvy = nullptr,
-      *gxbar = nullptr;
+    T *RX = nullptr, *RY = nullptr, *gx = nullptr, *gy = nullptr, *gvx = nullptr, *gvy = nullptr;
+    double2 *P = nullptr, *Q = nullptr;
+    const int S = std::min(kGSteps, ckpt);   // reverse steps packed together
     uint8_t *RMX = nullptr, *RMY = nullptr;
     double *ddc = nullptr, *ddq = nullptr, *ddv = nullptr;
     LP_TRY(B.alloc((void**)&RX, sizeof(T) * (size_t)(ckpt + 1) * n));
@@ -327,9 +404,10 @@ lp_status grad_impl(Handle* h, const lp_opts* o, int K, int ckpt, const double* 
     LP_TRY(B.alloc((void**)&RMY, (size_t)ckpt * m));
     LP_TRY(B.alloc((void**)&gx, sizeof(T) * n));
     LP_TRY(B.alloc((void**)&gy, sizeof(T) * m));
-    LP_TRY(B.alloc((void**)&gvx, sizeof(T) * n));
-    LP_TRY(B.alloc((void**)&gvy, sizeof(T) * m));
-    LP_TRY(B.alloc((void**)&gxbar, sizeof(T) * n));
+    LP_TRY(B.alloc((void**)&gvx, sizeof(T) * (size_t)S * n));
+    LP_TRY(B.alloc((void**)&gvy, sizeof(T) * (size_t)S * m));
+    LP_TRY(B.alloc((void**)&P, sizeof(double2) * (size_t)S * n));
+    LP_TRY(B.alloc((void**)&Q, sizeof(double2) * (size_t)S * m));
     LP_TRY(B.alloc((void**)&ddc, sizeof(double) * n));
     LP_TRY(B.alloc((void**)&ddq, sizeof(double) * m));
     LP_TRY(B.alloc((void**)&ddv, sizeof(double) * (size_t)std::max<int64_t>(nnz, 1)));
@@ -355,30 +433,38 @@ lp_status grad_impl(Handle* h, const lp_opts* o, int K, int ckpt, const double* 
                                     cudaMemcpyDeviceToDevice, st));
         LP_CUDA_TRY(cudaMemcpyAsync(RY, CY + (size_t)sgi * m, sizeof(T) * m,
                                     cudaMemcpyDeviceToDevice, st));
-        LP_TRY(products<T>(h, E, RX, RY, E.KX[0], E.KTY[0]));
+        LP_TRY(product<T>(h, E, RX, E.KX[0]));
         int c = 0;
         for (int s = 0; s < len; ++s) {
-            forward_step<T>(h, E, coef, RX + (size_t)s * n, RY + (size_t)s * m, E.KX[c], E.KTY[c],
+            forward_step<T>(h, E, coef, RX + (size_t)s * n, RY + (size_t)s * m, E.KX[c],
                             RX + (size_t)(s + 1) * n, RY + (size_t)(s + 1) * m, E.KX[c ^ 1],
-                            E.KTY[c ^ 1], RMX + (size_t)s * n, RMY + (size_t)s * m);
+                            RMX + (size_t)s * n, RMY + (size_t)s * m);
             c ^= 1;
         }
-        // reverse through the segment
-        for (int s = len - 1; s >= 0; --s) {
-            const T* xs = RX + (size_t)s * n;
-            const T* xs1 = RX + (size_t)(s + 1) * n;
-            const T* ys = RY + (size_t)s * m;
-            k_g_gvy<T><<<ew_grid_g(m), kEW, 0, st>>>(RMY + (size_t)s * m, gy, coef, gvy, ddq, m);
-            EpiStore<T> eg{gvy, gxbar, coef + 2, nullptr, nullptr};
+        // reverse through the segment; slot k of gvx and gvy: step s of the pack begun
+        // at step s + k
+        k_g_gvy<T><<<ew_grid_g(m), kEW, 0, st>>>(RMY + (size_t)(len - 1) * m, gy, coef, gvy, ddq, m);
+        ++h->launches;
+        for (int s = len - 1, k = 0; s >= 0; --s) {
+            const T* gvy_s = gvy + (size_t)k * m;
+            T* gvx_s = gvx + (size_t)k * n;
+            EpiGvx<T> eg{gvy_s, RMX + (size_t)s * n, coef, gx, gvx_s, ddc};
             launch_product<T>(h, E, true, st, eg);
-            k_g_gvx<T><<<ew_grid_g(n), kEW, 0, st>>>(RMX + (size_t)s * n, gx, gxbar, coef, gvx, ddc,
-                                                    n);
-            EpiGy<T> ey{gvx, gvy, coef, gy};
+            const bool full = ++k == S || s == 0;
+            // before the K product, which may write the first slot anew
+            if (full && nnz > 0) {
+                const int t = s + k - 1;
+                k_g_pack<T><<<ew_grid_g(n + m), kEW, 0, st>>>(k, S, RX + (size_t)t * n,
+                                                              RY + (size_t)t * m, gvx, gvy, coef, P, Q,
+                                                              n, m);
+                k_g_sddmm<<<ew_grid_g(nnz), kEW, 0, st>>>(h->krow, h->ci, P, Q, k, S, ddv, nnz);
+                h->launches += 2;
+            }
+            if (full) k = 0;
+            EpiGy<T> ey{gvx_s, gvy_s, coef, gy, s > 0 ? RMY + (size_t)(s - 1) * m : nullptr,
+                        gvy + (size_t)k * m, ddq};
             launch_product<T>(h, E, false, st, ey);
-            if (nnz > 0)
-                k_g_sddmm<T><<<ew_grid_g(nnz), kEW, 0, st>>>(h->krow, h->ci, gvy, gvx, xs, xs1, ys,
-                                                             coef, ddv, nnz);
-            h->launches += 5;
+            h->launches += 2;
         }
         LP_CUDA_TRY(cudaGetLastError());
     }

@@ -568,31 +568,4 @@ __device__ __forceinline__ void res_phase(const ResTile<T>& A, const ResVec<T, S
     (void)res_phase<T, SM>(A, x, f, product, [] { return true; });
 }
 
-// v clamped to [lo, hi] (l <= u; a NaN stays).  FP64: on the bit patterns as
-// integers, which order like the values (a sign bit turns the order round): an
-// FP64 comparison would take the FP64 unit.
-__device__ __forceinline__ double res_clamp(double v, double lo, double hi)
-{
-    const long long k = order_key(v);
-    const bool nan = (unsigned long long)(__double_as_longlong(v) & 0x7fffffffffffffffll) >
-                     0x7ff0000000000000ull;
-    double r = v;
-    if (k < order_key(lo)) r = lo;
-    if (k > order_key(hi)) r = hi;
-    return nan ? v : r;
-}
-__device__ __forceinline__ float res_clamp(float v, float lo, float hi)
-{
-    if (v < lo) v = lo;
-    if (v > hi) v = hi;
-    return v;
-}
-// v where it is not negative, else 0 (a NaN stays)
-__device__ __forceinline__ double res_pos(double v)
-{
-    const unsigned long long b = (unsigned long long)__double_as_longlong(v);
-    return b > 0x8000000000000000ull && b <= 0xfff0000000000000ull ? 0.0 : v;
-}
-__device__ __forceinline__ float res_pos(float v) { return v < 0.0f ? 0.0f : v; }
-
 }  // namespace pdhg
