@@ -194,7 +194,8 @@ __global__ void k_g_pack(int cnt, int stride, const T* X, const T* Y, const T* g
 // the packed steps one after the other.  A step by itself took five gathers of a 32-byte
 // sector, 32 bytes of indices and sums, and seven FP64 instructions a nonzero; eight packed
 // steps gather two 128-byte lines and take three instructions a step.  (Two, with the
-// steps' terms added up before they meet dA, lost a third of the last digits.)
+// steps' terms added up before they meet dA, were 1 % faster a call, with an error against
+// 64 bits of 1.3e-14 instead of 1.1e-14.)
 __global__ void k_g_sddmm(const int32_t* krow, const int32_t* ci, const double2* P, const double2* Q,
                           int cnt, int stride, double* dvals, int64_t nnz)
 {
