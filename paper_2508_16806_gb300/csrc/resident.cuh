@@ -238,7 +238,7 @@ struct __align__(16) ResPay {
 // Shared state of the barriers.
 struct ResShared {
     uint64_t mbar[2];                  // cluster form: arrivals of the x and of the y parts
-    ResPay out;                        // this block's sums
+    ResPay out[2];                     // this block's sums, two sets used in turn
     ResPay in[2][kResMaxCluster];      // every block's sums, two sets used in turn
     double tot[4];
     unsigned long long clk;
@@ -253,11 +253,22 @@ struct ResShared {
 // for it: they go on with what does not depend on the decision (warp 0 has no
 // rows) and meet it at the caller's next __syncthreads.  When a wait runs out,
 // sh.failed is set (and the error flag).
+//
+// Why nothing is overwritten while it may still be read (cluster form): a block
+// that has passed barrier b has every block's arrival at b, so every block has
+// passed b - 1: it has received this block's words of b - 1 (their bulk copies have
+// read their source), decided on b - 1 and done its product after b - 1.  A block
+// may therefore write, for barrier b + 1, over what it last sent at barrier b - 1 or
+// before, here and in the others' memory.  The sums take the two sets in turn by deciding
+// barriers alone, so a set comes back after one deciding barrier at least, whether
+// plain barriers lie between (the iterations) or not (the last two of the power
+// iteration); the parts of x and of y are sent at every other barrier (`side`
+// alternates), which also keeps the phases of the two mbarriers apart.
 struct ResBarrier {
     ResShared& sh;
     ResSlot* slots;            // grid form: [2][gridDim.x]
     unsigned long long* arrived;   // grid form: arrivals at barriers without sums, ever
-    unsigned int seq;              // barriers met (grid form: those with sums)
+    unsigned int seq;              // deciding barriers met
     unsigned long long plain;      // arrivals awaited
     unsigned int par;          // parities of the mbarriers' next waits
     int* err;
@@ -314,12 +325,13 @@ struct ResBarrier {
             return;
         }
         if (cluster) {
-            ++seq;
+            if (DEC) ++seq;
             ResPay* in = sh.in[seq & 1];
+            ResPay& out = sh.out[seq & 1];
             const uint32_t mb = res_smem(&sh.mbar[side]);
-            if (NV > 0 && warp < NV && lane == 0) sh.out.v[warp] = in[blockIdx.x].v[warp] = mine;
+            if (NV > 0 && warp < NV && lane == 0) out.v[warp] = in[blockIdx.x].v[warp] = mine;
             if (CLOCK && warp == 0 && lane == 0 && blockIdx.x == 0)
-                sh.out.clk = in[0].clk = global_ns();
+                out.clk = in[0].clk = global_ns();
             // this thread's entries are in the copy before the bulk copies read it
             asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
             __syncthreads();
@@ -335,7 +347,7 @@ struct ResBarrier {
                     const uint32_t src = res_smem(vec) + (uint32_t)blockIdx.x * (uint32_t)chunk;
                     res_bulk(res_mapa(src, lane), src, (uint32_t)chunk, rm);
                     if (DEC)
-                        res_bulk(res_mapa(res_smem(&in[blockIdx.x]), lane), res_smem(&sh.out), 32u, rm);
+                        res_bulk(res_mapa(res_smem(&in[blockIdx.x]), lane), res_smem(&out), 32u, rm);
                 }
             }
             const uint32_t want = (par >> side) & 1u;
