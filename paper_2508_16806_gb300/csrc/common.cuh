@@ -218,6 +218,11 @@ struct SlicedSide {
     // place of each LP [B + 1]
     const int32_t *tag = nullptr, *lp = nullptr, *lp0 = nullptr;
     double* part = nullptr;
+    // a batch: the slices of the LPs that were not done at the last check, as slice and tag
+    // ([nslice] each), and {their number, the finished LPs they were made for}
+    int4* slice_live = nullptr;
+    int32_t* tag_live = nullptr;
+    int* live = nullptr;
     const int32_t* row = nullptr;     // rows of the slices (-1: none)
     const int32_t* idx = nullptr;     // column of each entry (-1: padding)
     const int32_t* perm = nullptr;    // its nonzero

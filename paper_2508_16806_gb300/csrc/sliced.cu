@@ -173,6 +173,9 @@ lp_status slice_side(Handle* h, const std::vector<int64_t>& hrp, const int64_t* 
         LP_TRY(dev_alloc_n(h, &dlp, (size_t)ns));
         LP_TRY(dev_alloc_n(h, &dlp0, B + 1));
         LP_TRY(dev_alloc_n(h, &S.part, 2 * (size_t)ns));
+        LP_TRY(dev_alloc_n(h, &S.slice_live, (size_t)ns));
+        LP_TRY(dev_alloc_n(h, &S.tag_live, (size_t)ns));
+        LP_TRY(dev_alloc_n(h, &S.live, 2));
         LP_CUDA_TRY(cudaMemcpyAsync(dtag, tag.data(), (size_t)ns * 4, cudaMemcpyHostToDevice, st));
         LP_CUDA_TRY(cudaMemcpyAsync(dlp, lp.data(), (size_t)ns * 4, cudaMemcpyHostToDevice, st));
         LP_CUDA_TRY(cudaMemcpyAsync(dlp0, lps.data(), (B + 1) * 4, cudaMemcpyHostToDevice, st));

@@ -120,27 +120,31 @@ k_sliced(const SlicedSide S, const T* __restrict__ val, Epi epi)
 }
 
 // The same for a batch: a slice lies within one LP, whose state the epilogue takes
-// (and whose finish skips it); its partials go to the slice's place in row order.
+// (and whose finish skips it); its partials go to the slice's place in row order, so
+// they are the same bits from whichever list the slice comes.  live: the list of the
+// unfinished LPs instead of the whole one.
 template <typename T, class Epi>
 __global__ void __launch_bounds__(kSpmvNT, kSliceBlocks<T>)
-k_sliced_lp(const SlicedSide S, const T* __restrict__ val, Epi epi)
+k_sliced_lp(const SlicedSide S, const T* __restrict__ val, Epi epi, bool live)
 {
     typename Epi::Acc acc;
-    const int nw = gridDim.x * (kSpmvNT / 32), s1 = S.nslice;
+    const int4* __restrict__ rec = live ? S.slice_live : S.slice;
+    const int32_t* __restrict__ tag = live ? S.tag_live : S.tag;
+    const int nw = gridDim.x * (kSpmvNT / 32), s1 = live ? __ldg(S.live) : S.nslice;
     int s = (threadIdx.x >> 5) * gridDim.x + blockIdx.x;
     int4 d = make_int4(0, 0, 0, 0);
     int t = 0;
     if (s < s1) {
-        d = __ldg(S.slice + s);
-        t = __ldg(S.tag + s);
+        d = __ldg(rec + s);
+        t = __ldg(tag + s);
     }
     while (s < s1) {
         s += nw;
         int4 dn = d;
         int tn = t;
         if (s < s1) {
-            dn = __ldg(S.slice + s);
-            tn = __ldg(S.tag + s);
+            dn = __ldg(rec + s);
+            tn = __ldg(tag + s);
         }
         if (epi.live(t)) {
             epi.task_start(t);
