@@ -16,7 +16,7 @@ CSRC = os.path.join(HERE, "csrc")
 LIB = os.path.join(CSRC, "libpdhg.so")
 SOURCES = ["setup.cu", "solver.cu", "capi.cu", "grad.cu", "noalloc.cu", "batch.cu", "fishnet.cu",
            "tune.cu", "probe.cu", "resident.cu", "sliced.cu"]
-HEADERS = ["common.cuh", "spmv.cuh", "control.cuh", "resident.cuh", "sliced.cuh"]
+HEADERS = ["arith.cuh", "common.cuh", "spmv.cuh", "control.cuh", "resident.cuh", "sliced.cuh"]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 FLAGS = ["-O3", "-lineinfo", "-std=c++17", "-Xcompiler", "-fPIC", "-Xcompiler", "-O2"]
 

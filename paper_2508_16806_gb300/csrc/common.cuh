@@ -9,6 +9,7 @@
 #include <vector>
 
 #include "../../include/lp.h"
+#include "arith.cuh"
 
 namespace pdhg {
 
@@ -416,11 +417,10 @@ __device__ __forceinline__ double warp_sums16(double (&v)[16])
     return v[0] + __shfl_xor_sync(0xffffffffu, v[0], 16);
 }
 
-// Maximum of non-negative values over the warp (as integers, which order like
-// them; a NaN counts as the largest).
+// Maximum of non-negative values over the warp, as integers (nonneg_key).
 __device__ __forceinline__ double warp_max_nonneg(double v)
 {
-    unsigned long long b = (unsigned long long)__double_as_longlong(v);
+    unsigned long long b = nonneg_key(v);
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) {
         const unsigned long long u = __shfl_xor_sync(0xffffffffu, b, o);
