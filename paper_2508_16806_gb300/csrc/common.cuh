@@ -19,8 +19,9 @@ constexpr int kNT = 256;          // threads of an SpMV row-block
 constexpr int kEW = 256;          // threads of an elementwise block
 constexpr int kEWGrid = 1216;     // elementwise grid cap: 152 SMs x 8 resident blocks
 constexpr int kCtlNT = 512;       // threads of a control (single-block) kernel
-constexpr int kCheckNT = 512;     // threads and largest grid of the KKT-check reductions: two
-constexpr int kCheckGrid = 304;   // blocks per SM (more blocks only add partial sums)
+constexpr int kCheckNT = 512;     // threads and largest grid of the KKT-check reductions: as many
+constexpr int kCheckGrid = 608;   // threads as kEWGrid blocks of kEW (FP32 sums of a thread stay
+                                  // as short), in half the partial sums
 // KKT-check reductions: row side 11 sums + 2 maxima, column side 15 sums + 1 maximum
 constexpr int kRowSums = 11, kRowMax = 2, kRowQ = kRowSums + kRowMax;
 constexpr int kColSums = 15, kColMax = 1, kColQ = kColSums + kColMax;
@@ -270,8 +271,8 @@ struct Engine {
                                // K^T launch's fused primal step): one per block of the K^T
                                // launch grid, then one per split row of its schedule
     size_t partD_cap = 0, partT_cap = 0;        // allocated entries
-    double* partR = nullptr;   // [kRowQ][kEWGrid]
-    double* partC = nullptr;   // [kColQ][kEWGrid]
+    double* partR = nullptr;   // [kRowQ][check_grid(m)]
+    double* partC = nullptr;   // [kColQ][check_grid(n)]
     Ctrl* ctrl = nullptr;
     lp_trace_rec* trace = nullptr;  // device trace ring
     long long trace_cap = 0;
