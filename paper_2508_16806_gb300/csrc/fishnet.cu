@@ -67,17 +67,21 @@ __device__ __forceinline__ void spmm_row_part(const int32_t* __restrict__ ci,
 // out[r, p] = sum_k val_k X[col_k, p] for the rows r of a CSR matrix; X is row major with
 // P columns (a power of two, 1..64).  P / V lanes take a row, V columns (16 bytes where
 // P allows) each, and walk its nonzeros in order, eight gathers in flight (past the end:
-// the last entry again, times zero).  What bounds it is the chain start -> column -> gather
-// -> epilogue and, for many columns, the L2 bytes of the gathers; so many rows at once and
-// few instructions each.  50,000 x 100,000 LP, 625,000 nonzeros, P from 32 to 2, averages: a
-// warp per row 34 us (K^T side) and 24 us (K side); so 12.6 us and 13.0 us,
-// a call 11.4 -> 7.9 ms.
-template <typename T, int V, class Epi>
+// the last entry again, times zero).  G sums per column, one for every G-th nonzero, added
+// up in pairs: 32 / P of them below 32 points, as where the lanes of a warp share a row (one sum
+// for up to 128 nonzeros: up to 32 times as many roundings in a chain; FP64 steps, 50,000
+// rows, 64 points and fewer: 1,037 us instead of 1,090, FP32 289 instead of 288).
+// What bounds it is the chain start -> column -> gather -> epilogue and, for many columns,
+// the L2 bytes of the gathers; so many rows at once and few instructions each.  50,000 x
+// 100,000 LP, 625,000 nonzeros, P from 32 to 2, averages: a warp per row 34 us (K^T side)
+// and 24 us (K side); so 12.6 us and 13.0 us, a call 11.4 -> 7.9 ms.
+template <typename T, int V, int G, class Epi>
 __global__ void __launch_bounds__(kFW * 32)
 k_spmm(const int64_t* __restrict__ rp, const int32_t* __restrict__ ci,
        const T* __restrict__ val, int64_t rows, int P, const T* __restrict__ X, Epi epi)
 {
     using W = Vec<T, V>;
+    constexpr int S = G < 8 ? 8 : G;    // nonzeros of a round
     const int lr = P / V, per = kFW * 32 / lr;
     const int p = (int)(threadIdx.x & (lr - 1)) * V;
     for (int64_t r = (int64_t)blockIdx.x * per + threadIdx.x / lr; r < rows;
@@ -85,25 +89,39 @@ k_spmm(const int64_t* __restrict__ rp, const int32_t* __restrict__ ci,
         const int64_t s = rp[r], e = rp[r + 1];
         if (e - s > kLongRow) continue;
         const auto pre = epi.template load<V>(r, p);
-        W a;
+        W a[G];
 #pragma unroll
-        for (int i = 0; i < V; ++i) a.v[i] = T(0);
-        for (int64_t k = s; k < e; k += 8) {
-            int c[8];
-            T v[8];
-            W x[8];
+        for (int g = 0; g < G; ++g)
 #pragma unroll
-            for (int u = 0; u < 8; ++u) c[u] = ci[k + u < e ? k + u : e - 1];
+            for (int i = 0; i < V; ++i) a[g].v[i] = T(0);
+        for (int64_t k0 = s; k0 < e; k0 += S) {
 #pragma unroll
-            for (int u = 0; u < 8; ++u) v[u] = val[k + u < e ? k + u : e - 1];
+            for (int h = 0; h < S; h += 8) {
+                const int64_t k = k0 + h;
+                if (h > 0 && k >= e) break;
+                int c[8];
+                T v[8];
+                W x[8];
 #pragma unroll
-            for (int u = 0; u < 8; ++u) x[u] = *reinterpret_cast<const W*>(X + (int64_t)c[u] * P + p);
+                for (int u = 0; u < 8; ++u) c[u] = ci[k + u < e ? k + u : e - 1];
 #pragma unroll
-            for (int u = 0; u < 8; ++u)
+                for (int u = 0; u < 8; ++u) v[u] = val[k + u < e ? k + u : e - 1];
 #pragma unroll
-                for (int i = 0; i < V; ++i) a.v[i] = fma(k + u < e ? v[u] : T(0), x[u].v[i], a.v[i]);
+                for (int u = 0; u < 8; ++u) x[u] = *reinterpret_cast<const W*>(X + (int64_t)c[u] * P + p);
+#pragma unroll
+                for (int u = 0; u < 8; ++u)
+#pragma unroll
+                    for (int i = 0; i < V; ++i)
+                        a[(h + u) % G].v[i] = fma(k + u < e ? v[u] : T(0), x[u].v[i], a[(h + u) % G].v[i]);
+            }
         }
-        epi.template row<V>(r, p, a, pre);
+#pragma unroll
+        for (int o = 1; o < G; o <<= 1)
+#pragma unroll
+            for (int g = 0; g < G; g += 2 * o)
+#pragma unroll
+                for (int i = 0; i < V; ++i) a[g].v[i] += a[g + o].v[i];
+        epi.template row<V>(r, p, a[0], pre);
     }
 }
 
@@ -354,12 +372,15 @@ void spmm(Handle* h, const int64_t* rp, const int32_t* ci, const T* val, int64_t
     const int V = P < W ? P : W;
     const int64_t per = kFW * 32 / (P / V);
     const int grid = (int)std::max<int64_t>(1, std::min<int64_t>((rows + per - 1) / per, kFGrid));
-    if (V == 4)
-        k_spmm<T, W, Epi><<<grid, kFW * 32, 0, h->stream>>>(rp, ci, val, rows, P, X, epi);
-    else if (V == 2)
-        k_spmm<T, 2, Epi><<<grid, kFW * 32, 0, h->stream>>>(rp, ci, val, rows, P, X, epi);
-    else
-        k_spmm<T, 1, Epi><<<grid, kFW * 32, 0, h->stream>>>(rp, ci, val, rows, P, X, epi);
+    const auto go = [&](auto kernel) {
+        kernel<<<grid, kFW * 32, 0, h->stream>>>(rp, ci, val, rows, P, X, epi);
+    };
+    if (P >= 32) go(k_spmm<T, W, 1, Epi>);
+    else if (P == 16) go(k_spmm<T, W, 2, Epi>);
+    else if (P == 8) go(k_spmm<T, W, 4, Epi>);
+    else if (P == 4) go(k_spmm<T, W, 8, Epi>);
+    else if (P == 2) go(k_spmm<T, 2, 16, Epi>);
+    else go(k_spmm<T, 1, 32, Epi>);
     ++h->launches;
     if (nlong > 0) {
         k_spmm_long<T, Epi><<<std::min(nlong, kFGrid), kFW * 32, 0, h->stream>>>(
