@@ -27,9 +27,24 @@ namespace {
 constexpr int kFW = 8;             // warps per block of the block-SpMM kernels
 constexpr int kFGrid = 152 * 16;   // grid cap of the block-SpMM kernels (persistent rows loop)
 
-// Rows with more nonzeros than this go to k_spmm_long (a block per row), so that
-// no lane walks a power-law row of thousands of nonzeros alone.
-constexpr int64_t kLongRow = 128;
+// A side of up to kWarpRows rows, or of more than kLaneAvg nonzeros a row on average, takes
+// a warp per row (k_spmm_warp), any other lanes (k_spmm).  Products of all rounds of a step
+// from 2 / from 64 points down, us, warp | lanes.  Few rows, 12.5 nonzeros a row of K and 6.25
+// of K^T: FP64, 500 x 1,000 7.6 / 124 | 18.3 / 187, 2,000 x 4,000 13.2 / 164 | 21.6 / 206, the
+// K side of 5,000 rows 18.6 / 250 | 22.1 / 260, of 8,000 rows 20.4 / 317 | 22.4 / 303; FP32,
+// 500 rows 8.0 / 104 | 10.3 / 102, 2,000 10.1 / 114 | 11.5 / 116, the K side of 5,000
+// 12.1 / 128 | 12.2 / 125.  Long rows: 4,000 x 8,000, 129 to 256 a row, FP32 19.9 / 391 |
+// 34.7 / 508; 30,000 x 60,000, 80 a row, the K side 39.7 / 653 | 40.6 / 561, FP64 72 / 2,695 |
+// 61 / 2,075; 50,000 x 100,000, 40 a row, FP32 48 / 791 | 38 / 478.
+constexpr int64_t kLaneAvg = 48;
+template <typename T> constexpr int64_t kWarpRows = sizeof(T) == 4 ? 4096 : 6144;
+
+// Rows with more nonzeros than this go to k_spmm_long (a block per row), so that no lane
+// (kLaneRow) and no warp (kWarpRow) walks a power-law row of thousands of nonzeros alone.
+// kLaneRow at 64 | 128, the same figures, FP32: power-law rows of 4 to 2,000 35.0 / 678 |
+// 35.2 / 676, 1 % of the rows with 80 to 100 23.8 / 369 | 23.1 / 351, all with 80
+// 42.9 / 727 | 39.7 / 653; 2 % with 129 to 256 by lanes 34 / 505, by blocks 25 / 414.
+constexpr int64_t kLaneRow = 128, kWarpRow = 256;
 
 // V consecutive columns of a point block's row
 template <typename T, int V>
@@ -68,7 +83,7 @@ __device__ __forceinline__ void spmm_row_part(const int32_t* __restrict__ ci,
 // P columns (a power of two, 1..64).  P / V lanes take a row, V columns (16 bytes where
 // P allows) each, and walk its nonzeros in order, eight gathers in flight (past the end:
 // the last entry again, times zero).  G sums per column, one for every G-th nonzero, added
-// up in pairs: 32 / P of them below 32 points, as where the lanes of a warp share a row (one sum
+// up in pairs: 32 / P of them below 32 points, the sums of k_spmm_warp to the bit (one sum
 // for up to 128 nonzeros: up to 32 times as many roundings in a chain; FP64 steps, 50,000
 // rows, 64 points and fewer: 1,037 us instead of 1,090, FP32 289 instead of 288).
 // What bounds it is the chain start -> column -> gather -> epilogue and, for many columns,
@@ -87,32 +102,44 @@ k_spmm(const int64_t* __restrict__ rp, const int32_t* __restrict__ ci,
     for (int64_t r = (int64_t)blockIdx.x * per + threadIdx.x / lr; r < rows;
          r += (int64_t)gridDim.x * per) {
         const int64_t s = rp[r], e = rp[r + 1];
-        if (e - s > kLongRow) continue;
+        if (e - s > kLaneRow) continue;
         const auto pre = epi.template load<V>(r, p);
         W a[G];
 #pragma unroll
         for (int g = 0; g < G; ++g)
 #pragma unroll
             for (int i = 0; i < V; ++i) a[g].v[i] = T(0);
+        // FP32: the columns and values of the next eight are fetched while eight are gathered
+        // (10,000 x 20,000, 64 points and fewer: 167 -> 135 us; FP64 is bound by its unit
+        // instead, and slower so: 50,000 rows 1,090 -> 1,165 us)
+        constexpr bool AHEAD = sizeof(T) == 4;
+        int c[8];
+        T v[8];
+        const auto fetch = [&](int64_t k) {
+#pragma unroll
+            for (int u = 0; u < 8; ++u) c[u] = ci[k + u < e ? k + u : e - 1];
+#pragma unroll
+            for (int u = 0; u < 8; ++u) v[u] = k + u < e ? val[k + u] : T(0);
+        };
+        if (AHEAD && s < e) fetch(s);
         for (int64_t k0 = s; k0 < e; k0 += S) {
 #pragma unroll
             for (int h = 0; h < S; h += 8) {
                 const int64_t k = k0 + h;
                 if (h > 0 && k >= e) break;
-                int c[8];
-                T v[8];
                 W x[8];
-#pragma unroll
-                for (int u = 0; u < 8; ++u) c[u] = ci[k + u < e ? k + u : e - 1];
-#pragma unroll
-                for (int u = 0; u < 8; ++u) v[u] = val[k + u < e ? k + u : e - 1];
+                T w[8];
+                if (!AHEAD) fetch(k);
 #pragma unroll
                 for (int u = 0; u < 8; ++u) x[u] = *reinterpret_cast<const W*>(X + (int64_t)c[u] * P + p);
+#pragma unroll
+                for (int u = 0; u < 8; ++u) w[u] = v[u];
+                if (AHEAD && k + 8 < e) fetch(k + 8);
 #pragma unroll
                 for (int u = 0; u < 8; ++u)
 #pragma unroll
                     for (int i = 0; i < V; ++i)
-                        a[(h + u) % G].v[i] = fma(k + u < e ? v[u] : T(0), x[u].v[i], a[(h + u) % G].v[i]);
+                        a[(h + u) % G].v[i] = fma(w[u], x[u].v[i], a[(h + u) % G].v[i]);
             }
         }
 #pragma unroll
@@ -125,7 +152,35 @@ k_spmm(const int64_t* __restrict__ rp, const int32_t* __restrict__ ci,
     }
 }
 
-// The rows longer than kLongRow (listed in `rows`): one block per row, warp w
+// The same sums with a warp per row: lane l serves column l % P (and l + 32 when P = 64),
+// the G = 32 / P lane groups take every G-th nonzero of each batch of 32.  A row's columns
+// and values come in one load and its sums take few instructions of the FP64 unit: the
+// better form while a wave of warps holds the rows, and for long ones.
+template <typename T, class Epi>
+__global__ void __launch_bounds__(kFW * 32)
+k_spmm_warp(const int64_t* __restrict__ rp, const int32_t* __restrict__ ci,
+            const T* __restrict__ val, int64_t rows, int P, const T* __restrict__ X, Epi epi)
+{
+    const int lane = threadIdx.x & 31;
+    const int Pl = P < 32 ? P : 32;
+    const int G = 32 / Pl;
+    const int g = lane / Pl, p = lane % Pl;
+    const bool two = P == 64;
+    for (int64_t r = (int64_t)blockIdx.x * kFW + (threadIdx.x >> 5); r < rows;
+         r += (int64_t)gridDim.x * kFW) {
+        const int64_t s = rp[r], e = rp[r + 1];
+        if (e - s > kWarpRow) continue;
+        T a0 = 0, a1 = 0;
+        spmm_row_part(ci, val, s, e, 32, P, X, lane, G, g, p, two, a0, a1);
+        for (int o = Pl; o < 32; o <<= 1) a0 += __shfl_xor_sync(0xffffffffu, a0, o);
+        if (g == 0) {
+            epi.template row<1>(r, p, Vec<T, 1>{{a0}}, epi.template load<1>(r, p));
+            if (two) epi.template row<1>(r, p + 32, Vec<T, 1>{{a1}}, epi.template load<1>(r, p + 32));
+        }
+    }
+}
+
+// The longest rows (listed in `rows`): one block per row, warp w
 // takes the row's batches w, w + kFW, ...; the warps' sums are added in warp
 // order (fixed) before the epilogue.
 template <typename T, class Epi>
@@ -354,37 +409,43 @@ int ew_blocks(int64_t count)
     return (int)g;
 }
 
-// Rows of a CSR orientation with more than kLongRow nonzeros (host).
-std::vector<int32_t> long_rows(const std::vector<int64_t>& rp)
-{
-    std::vector<int32_t> out;
-    for (size_t r = 0; r + 1 < rp.size(); ++r)
-        if (rp[r + 1] - rp[r] > kLongRow) out.push_back((int32_t)r);
-    return out;
-}
+// The form of one side's products, and its rows that take a block each.
+template <typename T>
+struct Side {
+    bool warp;
+    std::vector<int32_t> rows;
+    int32_t* dev = nullptr;
+    explicit Side(const std::vector<int64_t>& rp)
+    {
+        const int64_t count = (int64_t)rp.size() - 1;
+        warp = count <= kWarpRows<T> || rp.back() > kLaneAvg * count;
+        for (int64_t r = 0; r < count; ++r)
+            if (rp[(size_t)r + 1] - rp[(size_t)r] > (warp ? kWarpRow : kLaneRow)) rows.push_back((int32_t)r);
+    }
+};
 
 // One block product: the short rows, then the long ones (a block each).
 template <typename T, class Epi>
 void spmm(Handle* h, const int64_t* rp, const int32_t* ci, const T* val, int64_t rows, int P,
-          const T* X, const int32_t* lrows, int nlong, const Epi& epi)
+          const T* X, const Side<T>& L, const Epi& epi)
 {
     constexpr int W = 16 / sizeof(T);   // columns of a 16-byte load
-    const int V = P < W ? P : W;
-    const int64_t per = kFW * 32 / (P / V);
+    const int64_t per = L.warp ? kFW : kFW * 32 / (P / (P < W ? P : W));   // rows of a block
     const int grid = (int)std::max<int64_t>(1, std::min<int64_t>((rows + per - 1) / per, kFGrid));
     const auto go = [&](auto kernel) {
         kernel<<<grid, kFW * 32, 0, h->stream>>>(rp, ci, val, rows, P, X, epi);
     };
-    if (P >= 32) go(k_spmm<T, W, 1, Epi>);
+    if (L.warp) go(k_spmm_warp<T, Epi>);
+    else if (P >= 32) go(k_spmm<T, W, 1, Epi>);
     else if (P == 16) go(k_spmm<T, W, 2, Epi>);
     else if (P == 8) go(k_spmm<T, W, 4, Epi>);
     else if (P == 4) go(k_spmm<T, W, 8, Epi>);
     else if (P == 2) go(k_spmm<T, 2, 16, Epi>);
     else go(k_spmm<T, 1, 32, Epi>);
     ++h->launches;
-    if (nlong > 0) {
-        k_spmm_long<T, Epi><<<std::min(nlong, kFGrid), kFW * 32, 0, h->stream>>>(
-            rp, ci, val, lrows, nlong, P, X, epi);
+    if (!L.rows.empty()) {
+        k_spmm_long<T, Epi><<<(int)std::min<size_t>(L.rows.size(), kFGrid), kFW * 32, 0, h->stream>>>(
+            rp, ci, val, L.dev, (int)L.rows.size(), P, X, epi);
         ++h->launches;
     }
 }
@@ -464,22 +525,18 @@ lp_status fishnet_t(Handle* h, double eta, double omega, double normK, int P, in
                                     cudaMemcpyHostToDevice, st));
         G = Gd;
     }
-    const std::vector<int32_t> lk = long_rows(h->h_rp), lt = long_rows(h->h_trp);
-    int32_t *lk_d = nullptr, *lt_d = nullptr;
-    LP_TRY(S.get(&lk_d, lk.size()));
-    LP_TRY(S.get(&lt_d, lt.size()));
-    if (!lk.empty())
-        LP_CUDA_TRY(cudaMemcpyAsync(lk_d, lk.data(), lk.size() * sizeof(int32_t),
-                                    cudaMemcpyHostToDevice, st));
-    if (!lt.empty())
-        LP_CUDA_TRY(cudaMemcpyAsync(lt_d, lt.data(), lt.size() * sizeof(int32_t),
-                                    cudaMemcpyHostToDevice, st));
-    const int nlk = (int)lk.size(), nlt = (int)lt.size();
+    Side<T> lk(h->h_rp), lt(h->h_trp);
+    for (Side<T>* q : {&lk, &lt}) {
+        LP_TRY(S.get(&q->dev, q->rows.size()));
+        if (!q->rows.empty())
+            LP_CUDA_TRY(cudaMemcpyAsync(q->dev, q->rows.data(), q->rows.size() * sizeof(int32_t),
+                                        cudaMemcpyHostToDevice, st));
+    }
     const T tau = (T)(eta / omega), sigma = (T)(eta * omega);
     // spectral casting, Y^0 = K~ X^0 (also the first K x)
     k_cast<T><<<ew_blocks(n * P), 256, 0, st>>>(n, P, normK / std::sqrt((double)n), G, X);
     ++h->launches;
-    spmm<T>(h, h->rp, h->ci, E.val, m, P, X, lk_d, nlk, FStore<T>{Y, P});
+    spmm<T>(h, h->rp, h->ci, E.val, m, P, X, lk, FStore<T>{Y, P});
     LP_CUDA_TRY(cudaMemcpyAsync(KX, Y, sizeof(T) * (size_t)m * P, cudaMemcpyDeviceToDevice, st));
     LP_CUDA_TRY(cudaGetLastError());
 
@@ -490,15 +547,15 @@ lp_status fishnet_t(Handle* h, double eta, double omega, double normK, int P, in
     while (cols > 1) {
         const int j_top = cols;
         for (int t = 0; t < k_steps; ++t) {
-            spmm<T>(h, h->trp, h->tci, E.tval, n, cols, Y, lt_d, nlt,
+            spmm<T>(h, h->trp, h->tci, E.tval, n, cols, Y, lt,
                     FPrimal<T>{X, Xn, E.c, E.l, E.u, tau, cols});
-            spmm<T>(h, h->rp, h->ci, E.val, m, cols, Xn, lk_d, nlk,
+            spmm<T>(h, h->rp, h->ci, E.val, m, cols, Xn, lk,
                     FDual<T>{Y, Yn, KX, E.q, h->sense, sigma, cols});
             std::swap(X, Xn);
             std::swap(Y, Yn);
         }
         // |duality gap| of every column
-        spmm<T>(h, h->trp, h->tci, E.tval, n, cols, Y, lt_d, nlt, FStore<T>{KTY, cols});
+        spmm<T>(h, h->trp, h->tci, E.tval, n, cols, Y, lt, FStore<T>{KTY, cols});
         k_gap_cols<T><<<nbC, kGapNT, 0, st>>>(n, cols, X, KTY, E.c, E.l, E.u, partC);
         k_gap_rows<T><<<nbR, kGapNT, 0, st>>>(m, cols, Y, E.q, partR);
         k_gap_final<<<cols, kGapNT, 0, st>>>(cols, partC, nbC, partR, nbR, gap);

@@ -1,5 +1,6 @@
 """Block products of fishnet casting with few points: a row's terms are added in 32 / P
-groups, whose sums then meet in pairs (csrc/fishnet.cu, k_spmm).
+groups, whose sums then meet in pairs, with a warp per row (few rows: k_spmm_warp in
+csrc/fishnet.cu) and with lanes (many: k_spmm) alike.
 
 Rows of 128 nonzeros, the first so large that a 1 added to it is lost, the others 1: the
 group of the first keeps it alone, every other group its 128 / G ones.  No steps: the dual
@@ -42,7 +43,7 @@ def test_groups_of_a_row(m, P, mixed):
 
 @pytest.mark.parametrize("P", [2, 4, 8, 16, 32, 64])
 def test_products_of_many_rows(oracle_mod, P):
-    """Every width and group count at the edges of its rounds of eight;
+    """Every width and group count of the lanes' form at the edges of its rounds of eight;
     bounds as in the other comparisons with the oracle: 1e-9 (FP64) and 1e-3 (FP32)."""
     torch = pytest.importorskip("torch")
     if not torch.cuda.is_available():
