@@ -78,6 +78,35 @@ __global__ void k_slice_values(int64_t entries, const int32_t* perm, const T* va
 
 }  // namespace
 
+// Whether a side's products are faster in slices than in the CSR ring (spmv.cuh), which
+// cuts long rows across warps and deals out nonzeros evenly.  steps: nonzeros of a lane if
+// all warps had the same.  A vector that L1 holds keeps the ring (its gathers hit there).
+//
+// The longest row: a slice takes it with 32 lanes, and the product waits for that warp.
+// Iterations (K and K^T) with one row of 20 | 2,048 | 4,096 | 8,000 nonzeros among rows of 5
+// to 20, us: FP64, 60,000 x 120,000 in slices 28 | 33 | 41 | 56, in the ring 41 for all;
+// 250,000 x 500,000 63 | 68 | 79 | 99 against 103; FP32, 100,000 x 200,000 24 | 24 | 34 | 48
+// against 24 | 24 | 29 | 30; 400,000 x 800,000 64 | 66 | 78 | 96 against 65 | 65 | 64 | 67.  The
+// 1M x 2M LP (rows of up to 5,000, 20M nonzeros) hides it: FP64 K side 220 -> 142 us, FP32
+// 116 -> 107.
+//
+// The average: FP64 slices were faster up to the 130 nonzeros a row that were tried (120,000
+// rows, ring -> slices: 20 a row 71 -> 47 us, 48 140 -> 75, 64 196 -> 93, 130 316 -> 155); the
+// line is at 48, above it nothing has moved.  FP32 gains little (1,000,000 rows of 12, K
+// side: 66.4 -> 63.7 us; 200,000 rows of 5 to 20: 26.5 -> 24.1) and loses where rows are
+// longer and warps few steps (100,000 rows of 22 to 66: 34.2 -> 36.5 us; the K^T side of
+// 150,000 rows of 20: 22.6 -> 24.7; with 300,000 rows of 22 to 66 72.7 -> 71.3).
+template <typename T>
+bool slices_pay(int64_t rows, int64_t nnz, int64_t maxrow, int64_t x_len, double steps, bool batch)
+{
+    const double avg = (double)nnz / (double)rows;
+    if (avg > 48.0 || maxrow > 8192 || x_len * (int64_t)sizeof(T) <= kL1GatherBytes) return false;
+    if (batch) return true;   // its ring cuts no rows
+    if (sizeof(T) == 4 && avg >= 16.0 && steps < 32.0) return false;
+    const double longest = (double)maxrow / 32.0;
+    return sizeof(T) == 4 ? longest <= std::max(64.0, 2.0 * steps) : longest <= std::max(128.0, 8.0 * steps);
+}
+
 template <typename T>
 lp_status slice_side(Handle* h, const std::vector<int64_t>& hrp, const int64_t* rp, const int32_t* ci,
                      int64_t x_len, const std::vector<int64_t>* lp0, SlicedSide* out)
@@ -86,16 +115,15 @@ lp_status slice_side(Handle* h, const std::vector<int64_t>& hrp, const int64_t* 
     SlicedSide S;
     *out = S;
     const int64_t rows = (int64_t)hrp.size() - 1, nnz = h->nnz;
-    // Long rows keep the CSR form, which cuts them across warps where its lists would be
-    // unbalanced; so does a vector that L1 holds (its gathers hit there)
-    if (nnz == 0 || (double)nnz > 48.0 * (double)rows) return LP_OK;
+    if (nnz == 0 || rows >= ((int64_t)1 << 31)) return LP_OK;
     int64_t maxrow = 0;
     for (int64_t r = 0; r < rows; ++r) maxrow = std::max(maxrow, hrp[(size_t)r + 1] - hrp[(size_t)r]);
-    if (maxrow > 8192 || x_len * (int64_t)sizeof(T) <= kL1GatherBytes || rows >= ((int64_t)1 << 31))
-        return LP_OK;
     cudaStream_t st = h->stream;
     int sms = 0;
     LP_CUDA_TRY(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, h->device));
+    if (!slices_pay<T>(rows, nnz, maxrow, x_len,
+                       (double)nnz / 32.0 / (double)(sms * kSliceBlocks<T> * (kSpmvNT / 32)), lp0 != nullptr))
+        return LP_OK;
     // windows of W rows, none across two LPs
     const size_t B = lp0 ? lp0->size() - 1 : 1;
     std::vector<int32_t> wst, wfirst(B + 1);

@@ -1,4 +1,5 @@
-// Products with K and K^T in sliced rows: the form for short rows.
+// Products with K and K^T in sliced rows (SELL-C-sigma: Kreutzer et al., 2014): the form for
+// short rows.
 //
 // Rows are taken kSliceWin at a time, sorted by length, and cut into slices: 32
 // lanes that serve 32 / G rows with G lanes each (G = 1 up to kSliceRow nonzeros),
