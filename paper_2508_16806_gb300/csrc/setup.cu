@@ -350,19 +350,34 @@ __global__ void k_fill(T* p, int64_t count, T v)
 // order of products on both sides, so K^T stays the exact transpose of K.  NORMS: infinity
 // norms of the rows and their largest deviation |1 - norm| (non-empty rows) per LP.
 // Groups of 2^lg lanes take a row, four entries per lane in flight (past the end: the
-// lane's first entry again), the whole warp what is left of a row after 16 entries per lane.  Both sides hold their values, so no norm needs an atomic per
-// nonzero and no pass reads the matrix a second time; the maxima are of bit patterns (they
-// order like the non-negative values: an FP64 maximum costs 200 cycles of a warp here).
+// lane's first entry again), the whole warp what is left of a row after 16 entries per lane,
+// the whole block, when its rows are done, what is left of up to kRuizBig rows with more than
+// kRuizLong entries.  Both sides hold their values, so no norm needs an atomic per nonzero and
+// no pass reads the matrix a second time; the maxima are of bit patterns (they order like the
+// non-negative values: an FP64 maximum costs 200 cycles of a warp here).
 // Bound by the chain of a row's loads (start, entries, factors).  64 LPs stacked: the passes
 // of a solve, with an atomic per nonzero for the column norms (a warp per row 417 us) and
 // one per row for the deviation (902 us a pass), 14 -> 2 ms, a solve 58.2 -> 46.5 ms.  1M x
 // 2M LP with 20M power-law rows: 647 us a pass (830 us with lanes chosen for the longest row).
+// One long row among 100,000 short ones, us a pass, its rest by a warp -> by the block (an
+// atomic per nonzero): 20 nonzeros 59 -> 59 (141), 8,000 129 -> 60 (147), 20,000 250 -> 73
+// (174), 500,000 5,009 -> 617 (1,332).
+constexpr int kRuizBig = 32, kRuizLong = 1024;
+struct RuizRest {               // the rest of a row: its entries, its factor, the maximum so far
+    int64_t row, p, e;
+    double own;
+    unsigned long long mx;
+};
 template <bool SCALE, bool NORMS>
 __global__ void __launch_bounds__(kRuizNT)
 k_ruiz_pass(RuizSide a, RuizSide b, unsigned long long* dev)
 {
     __shared__ unsigned long long shd[kRuizNT / 32];
     __shared__ int shk[kRuizNT / 32];
+    __shared__ RuizRest big[kRuizBig];
+    __shared__ int nbig;
+    if (threadIdx.x == 0) nbig = 0;
+    __syncthreads();
     const bool tside = (int)blockIdx.x >= a.blocks;
     const RuizSide S = tside ? b : a;
     const int lg = S.lg, G = 1 << lg, per = kRuizNT >> lg;
@@ -421,6 +436,7 @@ k_ruiz_pass(RuizSide a, RuizSide b, unsigned long long* dev)
             if (SCALE) on = S.own[row + per];
         }
         unsigned long long mx = 0;
+        int late = -1;          // the row's place among the block's
         for (int k = 0; k < 4 && p < e; ++k, p += 4 * G) {
             const unsigned long long t = take(p, e, G, own);
             mx = t > mx ? t : mx;
@@ -431,6 +447,16 @@ k_ruiz_pass(RuizSide a, RuizSide b, unsigned long long* dev)
             const int src = __ffs(rest) - 1;
             const int64_t p0 = __shfl_sync(0xffffffffu, p, src), e0 = __shfl_sync(0xffffffffu, e, src);
             const double o0 = __shfl_sync(0xffffffffu, own, src);
+            if (e0 - p0 > kRuizLong) {
+                int k = 0;
+                if (lane == src) k = atomicAdd(&nbig, 1);
+                k = __shfl_sync(0xffffffffu, k, src);
+                if (k < kRuizBig) {
+                    if (lane - g == src) late = k;
+                    if (lane == src) big[k] = RuizRest{row, p0, e0, o0, 0};
+                    continue;
+                }
+            }
             unsigned long long t = 0;
             for (int64_t pp = p0 + lane; pp < e0; pp += 128) {
                 const unsigned long long t1 = take(pp, e0, 32, o0);
@@ -447,7 +473,9 @@ k_ruiz_pass(RuizSide a, RuizSide b, unsigned long long* dev)
                 const unsigned long long t = __shfl_xor_sync(0xffffffffu, mx, o);
                 mx = t > mx ? t : mx;
             }
-            if (in) {
+            if (late >= 0) {
+                if (g == 0) big[late].mx = mx;
+            } else if (in) {
                 const double nr = __longlong_as_double((long long)mx);
                 if (g == 0) S.nrm[row] = nr;
                 const int k = S.lp ? S.lp[row] : 0;
@@ -459,6 +487,33 @@ k_ruiz_pass(RuizSide a, RuizSide b, unsigned long long* dev)
                 const unsigned long long t = (unsigned long long)__double_as_longlong(fabs(1.0 - nr));
                 if (mx != 0 && t > dm) dm = t;
             }
+        }
+    }
+    // the long rows, by the whole block
+    __syncthreads();
+    for (int i = 0; i < min(nbig, kRuizBig); ++i) {
+        const RuizRest R = big[i];
+        unsigned long long mx = 0;
+        for (int64_t p = R.p + threadIdx.x; p < R.e; p += 4 * kRuizNT) {
+            const unsigned long long t = take(p, R.e, kRuizNT, R.own);
+            mx = t > mx ? t : mx;
+        }
+        if (NORMS) {
+            for (int o = 16; o > 0; o >>= 1) {
+                const unsigned long long t = __shfl_xor_sync(0xffffffffu, mx, o);
+                mx = t > mx ? t : mx;
+            }
+            if (lane == 0) shd[threadIdx.x >> 5] = mx;
+            __syncthreads();
+            if (threadIdx.x == 0) {
+                mx = R.mx;
+                for (int w = 0; w < kRuizNT / 32; ++w) mx = shd[w] > mx ? shd[w] : mx;
+                const double nr = __longlong_as_double((long long)mx);
+                S.nrm[R.row] = nr;
+                const unsigned long long t = (unsigned long long)__double_as_longlong(fabs(1.0 - nr));
+                if (mx != 0 && t != 0) atomicMax(dev + (S.lp ? S.lp[R.row] : 0), t);
+            }
+            __syncthreads();
         }
     }
     if (NORMS) {
