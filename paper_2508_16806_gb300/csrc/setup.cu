@@ -1040,18 +1040,10 @@ static lp_status upload_split(Handle* h, const SplitPlan& plan, SplitRows& sp)
     return LP_OK;
 }
 
-// A side in sliced rows: its launch's blocks and partials.
+// Room for the partials of both sides' launches.
 template <typename T>
-static lp_status engine_grids(Handle* h, Engine<T>& E)
+static lp_status engine_partials(Handle* h, Engine<T>& E)
 {
-    if (E.slK.on) {
-        E.gK = E.npK = E.slK.grid;
-        E.splitK.n = 0;
-    }
-    if (E.slT.on) {
-        E.gT = E.npT = E.slT.grid;
-        E.splitT.n = 0;
-    }
     const size_t needD = 2 * (size_t)E.npK + 8, needT = std::max<size_t>((size_t)E.npT, (size_t)kEWGrid) + 8;
     if (needD > E.partD_cap) {
         dev_free(h, E.partD);
@@ -1068,33 +1060,45 @@ static lp_status engine_grids(Handle* h, Engine<T>& E)
     return LP_OK;
 }
 
-// Allocation, schedules and (for T = float) the FP32 casts of the scaled data.
+// The launches of one side: its blocks and partials and, unless its products run in slices,
+// the CSR ring's task lists.  (Built for sliced sides too, with the slices in five
+// allocations each, the first setup of a 200,000 x 400,000 LP with FP32 iterations took
+// 19.3 ms instead of 8.9, of a 60,000 x 120,000 LP 10.5 ms instead of 8.0.)
 template <typename T>
-lp_status engine_schedule(Handle* h, SchedParams sK, SchedParams sT)
+static lp_status schedule_side(Handle* h, bool side_t, SchedParams sp)
 {
     Engine<T>& E = engine_of<T>(h);
-    std::vector<int32_t> bk = make_row_blocks(h->h_rp.data(), h->m, sK.cap, sK.max_rows);
-    std::vector<int32_t> bt = make_row_blocks(h->h_trp.data(), h->n, sT.cap, sT.max_rows);
-    std::vector<int64_t> nk(bk.size()), nt(bt.size());
-    for (size_t t = 0; t < bk.size(); ++t) nk[t] = h->h_rp[(size_t)bk[t]];
-    for (size_t t = 0; t < bt.size(); ++t) nt[t] = h->h_trp[(size_t)bt[t]];
+    const std::vector<int64_t>& hrp = side_t ? h->h_trp : h->h_rp;
+    int32_t*& rows = side_t ? E.bcol : E.brow;
+    int64_t*& nz = side_t ? E.bnzT : E.bnzK;
+    int32_t*& wbeg = side_t ? E.wbegT : E.wbegK;
+    int32_t*& perm = side_t ? E.permT : E.permK;
+    SplitRows& split = side_t ? E.splitT : E.splitK;
+    int& ntask = side_t ? E.ntblk : E.nblk;
+    int& grid = side_t ? E.gT : E.gK;
+    int& np = side_t ? E.npT : E.npK;
+    for (void* p : {(void*)rows, (void*)nz, (void*)wbeg, (void*)perm}) dev_free(h, p);
+    rows = wbeg = perm = nullptr;
+    nz = nullptr;
+    const SlicedSide& S = side_t ? E.slT : E.slK;
+    if (S.on) {
+        LP_TRY(upload_split<T>(h, SplitPlan{}, split));
+        ntask = 0;
+        grid = np = S.grid;
+        return LP_OK;
+    }
+    std::vector<int32_t> b = make_row_blocks(hrp.data(), (int64_t)hrp.size() - 1, sp.cap, sp.max_rows);
+    std::vector<int64_t> first(b.size());
+    for (size_t t = 0; t < b.size(); ++t) first[t] = hrp[(size_t)b[t]];
     int sms = 0;
     LP_CUDA_TRY(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, h->device));
-    const int gK = spmv_grid<T>((int)bk.size() - 1, sms), gT = spmv_grid<T>((int)bt.size() - 1, sms);
-    // long rows cut into pieces where the lists would be unbalanced (the grids
-    // stay those of the uncut schedules)
-    const SplitPlan spK = split_long_rows(bk, nk, sK.cap, gK * kSpmvWorkers);
-    const SplitPlan spT = split_long_rows(bt, nt, sT.cap, gT * kSpmvWorkers);
-    std::vector<int32_t> wk, pk, wt, pt;
-    assign_tasks(nk, sK.cap, gK * kSpmvWorkers, wk, pk);
-    assign_tasks(nt, sT.cap, gT * kSpmvWorkers, wt, pt);
-    for (void* p : {(void*)E.brow, (void*)E.bcol, (void*)E.bnzK, (void*)E.bnzT, (void*)E.wbegK,
-                    (void*)E.permK, (void*)E.wbegT, (void*)E.permT})
-        dev_free(h, p);
-    E.brow = E.bcol = E.wbegK = E.permK = E.wbegT = E.permT = nullptr;
-    E.bnzK = E.bnzT = nullptr;
-    LP_TRY(upload_split<T>(h, spK, E.splitK));
-    LP_TRY(upload_split<T>(h, spT, E.splitT));
+    grid = spmv_grid<T>((int)b.size() - 1, sms);
+    // long rows cut into pieces where the lists would be unbalanced (the grid
+    // stays that of the uncut schedule)
+    const SplitPlan plan = split_long_rows(b, first, sp.cap, grid * kSpmvWorkers);
+    std::vector<int32_t> w, pm;
+    assign_tasks(first, sp.cap, grid * kSpmvWorkers, w, pm);
+    LP_TRY(upload_split<T>(h, plan, split));
     // Row sums of each short task: one group of lanes per row where that is
     // balanced, equal lane shares (seg_row_sums, with its fixed cost of a
     // search and a five-round scan) where the busiest lane would take more than
@@ -1104,52 +1108,37 @@ lp_status engine_schedule(Handle* h, SchedParams sK, SchedParams sT)
     // times an equal share; above 8 steps: K side 284 -> 249 us, K^T side
     // 202 -> 193 us).  In FP32 no threshold (16 to 48) was faster than none.
     const int seg_steps = sizeof(T) == 8 ? PDHG_SEG_STEPS_F64 : PDHG_SEG_STEPS_F32;
-    const std::vector<char> segK = seg_tasks(h->h_rp.data(), bk, nk, sK.cap, seg_steps);
-    const std::vector<char> segT = seg_tasks(h->h_trp.data(), bt, nt, sT.cap, seg_steps);
-    for (size_t t = 0; t < segK.size(); ++t)
-        if (segK[t]) nk[t] |= kSegBit;
-    for (size_t t = 0; t < segT.size(); ++t)
-        if (segT[t]) nt[t] |= kSegBit;
+    const std::vector<char> seg = seg_tasks(hrp.data(), b, first, sp.cap, seg_steps);
+    for (size_t t = 0; t < seg.size(); ++t)
+        if (seg[t]) first[t] |= kSegBit;
     // a piece carries its slot + 1 in the high 32 bits of its first nonzero
-    for (size_t t = 0; t < spK.task_piece.size(); ++t)
-        if (spK.task_piece[t] >= 0) nk[t] |= (int64_t)(spK.task_piece[t] + 1) << 32;
-    for (size_t t = 0; t < spT.task_piece.size(); ++t)
-        if (spT.task_piece[t] >= 0) nt[t] |= (int64_t)(spT.task_piece[t] + 1) << 32;
+    for (size_t t = 0; t < plan.task_piece.size(); ++t)
+        if (plan.task_piece[t] >= 0) first[t] |= (int64_t)(plan.task_piece[t] + 1) << 32;
     // step partials: one per block, then one per split row
-    E.npK = gK + spK.n;
-    E.npT = gT + spT.n;
-    LP_TRY(dev_alloc_n(h, &E.brow, bk.size()));
-    LP_TRY(dev_alloc_n(h, &E.bcol, bt.size()));
-    LP_TRY(dev_alloc_n(h, &E.bnzK, nk.size()));
-    LP_TRY(dev_alloc_n(h, &E.bnzT, nt.size()));
-    LP_TRY(dev_alloc_n(h, &E.wbegK, wk.size()));
-    LP_TRY(dev_alloc_n(h, &E.permK, pk.size()));
-    LP_TRY(dev_alloc_n(h, &E.wbegT, wt.size()));
-    LP_TRY(dev_alloc_n(h, &E.permT, pt.size()));
-    LP_CUDA_TRY(cudaMemcpyAsync(E.wbegK, wk.data(), wk.size() * sizeof(int32_t),
-                                cudaMemcpyHostToDevice, h->stream));
-    if (!pk.empty())
-        LP_CUDA_TRY(cudaMemcpyAsync(E.permK, pk.data(), pk.size() * sizeof(int32_t),
-                                    cudaMemcpyHostToDevice, h->stream));
-    LP_CUDA_TRY(cudaMemcpyAsync(E.wbegT, wt.data(), wt.size() * sizeof(int32_t),
-                                cudaMemcpyHostToDevice, h->stream));
-    if (!pt.empty())
-        LP_CUDA_TRY(cudaMemcpyAsync(E.permT, pt.data(), pt.size() * sizeof(int32_t),
-                                    cudaMemcpyHostToDevice, h->stream));
-    LP_CUDA_TRY(cudaMemcpyAsync(E.brow, bk.data(), bk.size() * sizeof(int32_t),
-                                cudaMemcpyHostToDevice, h->stream));
-    LP_CUDA_TRY(cudaMemcpyAsync(E.bcol, bt.data(), bt.size() * sizeof(int32_t),
-                                cudaMemcpyHostToDevice, h->stream));
-    LP_CUDA_TRY(cudaMemcpyAsync(E.bnzK, nk.data(), nk.size() * sizeof(int64_t),
-                                cudaMemcpyHostToDevice, h->stream));
-    LP_CUDA_TRY(cudaMemcpyAsync(E.bnzT, nt.data(), nt.size() * sizeof(int64_t),
-                                cudaMemcpyHostToDevice, h->stream));
+    np = grid + plan.n;
+    const auto up = [&](auto** d, const auto& v) -> lp_status {
+        LP_TRY(dev_alloc_n(h, d, v.size()));
+        if (!v.empty())
+            LP_CUDA_TRY(cudaMemcpyAsync(*d, v.data(), v.size() * sizeof(v[0]), cudaMemcpyHostToDevice,
+                                        h->stream));
+        return LP_OK;
+    };
+    LP_TRY(up(&rows, b));
+    LP_TRY(up(&nz, first));
+    LP_TRY(up(&wbeg, w));
+    LP_TRY(up(&perm, pm));
     LP_CUDA_TRY(cudaStreamSynchronize(h->stream));   // the host vectors go out of scope
-    E.nblk = (int)bk.size() - 1;
-    E.ntblk = (int)bt.size() - 1;
-    E.gK = gK;
-    E.gT = gT;
-    LP_TRY(engine_grids(h, E));
+    ntask = (int)b.size() - 1;
+    return LP_OK;
+}
+
+template <typename T>
+lp_status engine_schedule(Handle* h, SchedParams sK, SchedParams sT)
+{
+    Engine<T>& E = engine_of<T>(h);
+    LP_TRY(schedule_side<T>(h, false, sK));
+    LP_TRY(schedule_side<T>(h, true, sT));
+    LP_TRY(engine_partials(h, E));
     E.schedK = sK;
     E.schedT = sT;
     return LP_OK;
@@ -1158,6 +1147,7 @@ lp_status engine_schedule(Handle* h, SchedParams sK, SchedParams sT)
 template lp_status engine_schedule<double>(Handle*, SchedParams, SchedParams);
 template lp_status engine_schedule<float>(Handle*, SchedParams, SchedParams);
 
+// Allocation, the form of the products and (for T = float) the FP32 casts of the scaled data.
 template <typename T>
 lp_status setup_engine(Handle* h, const lp_opts* o)
 {
@@ -1165,6 +1155,8 @@ lp_status setup_engine(Handle* h, const lp_opts* o)
     const int64_t m = h->m, n = h->n, nnz = h->nnz;
     Engine<T>& E = engine_of<T>(h);
     if (!E.ready) {
+        LP_TRY(res_plan<T>(h));
+        if (!E.res.on) LP_TRY(slice_plan<T>(h));
         // the K side gathers x (n entries), the K^T side y (m entries)
         LP_TRY(engine_schedule<T>(h, SchedParams{spmv_cap<T>(n), kTaskRows},
                                   SchedParams{spmv_cap<T>(m), kTaskRows}));
@@ -1181,9 +1173,6 @@ lp_status setup_engine(Handle* h, const lp_opts* o)
         LP_TRY(dev_alloc_n(h, &E.partR, kRowQ * (size_t)kCheckGrid));
         LP_TRY(dev_alloc_n(h, &E.partC, kColQ * (size_t)kCheckGrid));
         LP_TRY(dev_alloc_n(h, &E.ctrl, 1));
-        LP_TRY(res_plan<T>(h));
-        if (!E.res.on) LP_TRY(slice_plan<T>(h));
-        LP_TRY(engine_grids(h, E));
         E.ready = true;
     }
     if (std::is_same<T, float>::value) {

@@ -135,10 +135,10 @@ lp_status slice_side(Handle* h, const std::vector<int64_t>& hrp, const int64_t* 
     const int nwin = wfirst[B] = (int32_t)wst.size();
     wst.push_back((int32_t)rows);
     std::vector<int4> w((size_t)nwin);
-    int4 *dw = nullptr, *raw = nullptr;
-    int32_t* dst = nullptr;
-    LP_TRY(dev_alloc_n(h, &dw, (size_t)nwin));
-    LP_TRY(dev_alloc_n(h, &dst, wst.size()));
+    // the windows' lists lie in the handle's scratch: 20 bytes for 128 rows and an LP, of
+    // 16 for every row and column
+    int4* dw = reinterpret_cast<int4*>(h->scratch);
+    int32_t* dst = reinterpret_cast<int32_t*>(dw + nwin);
     LP_CUDA_TRY(cudaMemcpyAsync(dst, wst.data(), wst.size() * 4, cudaMemcpyHostToDevice, st));
     k_slice_rows<W><<<nwin, W, 0, st>>>(dst, rp, dw, nullptr, nullptr, nullptr);
     LP_CUDA_TRY(cudaGetLastError());
@@ -157,17 +157,15 @@ lp_status slice_side(Handle* h, const std::vector<int64_t>& hrp, const int64_t* 
     LP_CUDA_TRY(cudaMemGetInfo(&avail, &total));
     const size_t need = (size_t)ns * sizeof(int4) + (size_t)nl * 4 + (size_t)steps * 32 * (8 + sizeof(T));
     if (steps * 32 >= ((int64_t)1 << 31) || nl >= ((int64_t)1 << 31) || need > avail / 4) {
-        dev_free(h, dw);
-        dev_free(h, dst);
         return LP_OK;
     }
-    int32_t *list = nullptr, *idx = nullptr, *perm = nullptr;
+    // one allocation: values, records, columns, nonzeros, rows
     T* val = nullptr;
-    LP_TRY(dev_alloc_n(h, &raw, (size_t)ns));
-    LP_TRY(dev_alloc_n(h, &list, (size_t)nl));
-    LP_TRY(dev_alloc_n(h, &idx, (size_t)steps * 32));
-    LP_TRY(dev_alloc_n(h, &perm, (size_t)steps * 32));
-    LP_TRY(dev_alloc_n(h, &val, (size_t)steps * 32));
+    LP_TRY(dev_alloc(h, (void**)&val, need));
+    int4* raw = reinterpret_cast<int4*>(val + steps * 32);
+    int32_t* idx = reinterpret_cast<int32_t*>(raw + ns);
+    int32_t* perm = idx + steps * 32;
+    int32_t* list = perm + steps * 32;
     LP_CUDA_TRY(cudaMemcpyAsync(dw, w.data(), (size_t)nwin * sizeof(int4), cudaMemcpyHostToDevice, st));
     k_slice_rows<W><<<nwin, W, 0, st>>>(dst, rp, nullptr, dw, raw, list);
     k_slice_fill<<<4 * 1216, 256, 0, st>>>((int)ns, raw, list, rp, ci, idx, perm);
@@ -212,8 +210,6 @@ lp_status slice_side(Handle* h, const std::vector<int64_t>& hrp, const int64_t* 
         S.lp0 = dlp0;
     }
     LP_CUDA_TRY(cudaStreamSynchronize(st));
-    dev_free(h, dw);
-    dev_free(h, dst);
     S.slice = raw;
     S.row = list;
     S.idx = idx;
