@@ -132,7 +132,9 @@ typedef struct {
                                     warp-task schedules of K and K^T (nonzeros and rows per task)
                                     on the device and keep the fastest of each (a candidate must
                                     beat the default by 3 %); the summation order, and so the
-                                    last bits of the result, then depends on that timing.
+                                    last bits of the result, then depends on that timing.  Sides
+                                    whose products run without such tasks (small LPs, short
+                                    rows) are left alone.
                                     0 (default): the largest tasks (the compiled defaults) */
     int32_t halpern;             /* 1: restarted (reflected) Halpern PDHG, the variant the
                                     Conclusion names as future work (Lu and Yang, 2024), in

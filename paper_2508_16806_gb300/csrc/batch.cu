@@ -859,15 +859,21 @@ lp_status tune_batch(BatchHandle* bh)
     LP_CUDA_TRY(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, h->device));
     LP_CUDA_TRY(cudaMemsetAsync(E.XA, 0, sizeof(T) * (size_t)h->n, h->stream));
     LP_CUDA_TRY(cudaMemsetAsync(E.YA, 0, sizeof(T) * (size_t)h->m, h->stream));
-    SchedParams pK, pT;
-    float msK = 0.0f, msT = 0.0f;
-    LP_TRY(tune_schedule<T>(
-        sms, h->stream, [&](int cap, int rows) { return batch_blocks(bh, true, {cap, rows}); },
-        h->h_rp.data(), h->rp, h->ci, E.val, E.XA, E.KXA, h->n, h->dev_err, &pK, &msK));
-    LP_TRY(tune_schedule<T>(
-        sms, h->stream, [&](int cap, int rows) { return batch_blocks(bh, false, {cap, rows}); },
-        h->h_trp.data(), h->trp, h->tci, E.tval, E.YA, E.KTYA, h->m, h->dev_err, &pT, &msT));
-    h->launches += 2 * 6 * 4;
+    // a side in slices runs no task lists but the checks', which are not worth a trial
+    SchedParams pK = S.pK, pT = S.pT;
+    float ms = 0.0f;
+    if (!S.slK.on) {
+        LP_TRY(tune_schedule<T>(
+            sms, h->stream, [&](int cap, int rows) { return batch_blocks(bh, true, {cap, rows}); },
+            h->h_rp.data(), h->rp, h->ci, E.val, E.XA, E.KXA, h->n, h->dev_err, &pK, &ms));
+        h->launches += 6 * 4;
+    }
+    if (!S.slT.on) {
+        LP_TRY(tune_schedule<T>(
+            sms, h->stream, [&](int cap, int rows) { return batch_blocks(bh, false, {cap, rows}); },
+            h->h_trp.data(), h->trp, h->tci, E.tval, E.YA, E.KTYA, h->m, h->dev_err, &pT, &ms));
+        h->launches += 6 * 4;
+    }
     if (pK.cap != S.pK.cap || pK.max_rows != S.pK.max_rows || pT.cap != S.pT.cap ||
         pT.max_rows != S.pT.max_rows) {
         LP_TRY(build_sched<T>(bh, pK, pT));

@@ -102,6 +102,8 @@ template lp_status tune_schedule<float>(int, cudaStream_t, const RowBlockBuilder
                                         const float*, const float*, float*, int64_t, int*,
                                         SchedParams*, float*);
 
+// The sides of an engine whose loop runs on task lists: neither resident iterations nor
+// slices do.
 template <typename T>
 lp_status tune_engine(Handle* h)
 {
@@ -113,17 +115,22 @@ lp_status tune_engine(Handle* h)
     // inputs: zeroed averages (scratch until the next check); outputs: their products
     LP_CUDA_TRY(cudaMemsetAsync(E.XA, 0, sizeof(T) * (size_t)n, h->stream));
     LP_CUDA_TRY(cudaMemsetAsync(E.YA, 0, sizeof(T) * (size_t)m, h->stream));
-    SchedParams sK, sT;
-    float msK = 0.0f, msT = 0.0f;
+    SchedParams sK = E.schedK, sT = E.schedT;
+    float ms = 0.0f;
     const int64_t* hrp = h->h_rp.data();
     const int64_t* htrp = h->h_trp.data();
-    LP_TRY(tune_schedule<T>(
-        sms, h->stream, [&](int cap, int rows) { return make_row_blocks(hrp, m, cap, rows); },
-        hrp, h->rp, h->ci, E.val, E.XA, E.KXA, n, h->dev_err, &sK, &msK));
-    LP_TRY(tune_schedule<T>(
-        sms, h->stream, [&](int cap, int rows) { return make_row_blocks(htrp, n, cap, rows); },
-        htrp, h->trp, h->tci, E.tval, E.YA, E.KTYA, m, h->dev_err, &sT, &msT));
-    h->launches += 2 * 6 * 4;
+    if (!E.res.on && !E.slK.on) {
+        LP_TRY(tune_schedule<T>(
+            sms, h->stream, [&](int cap, int rows) { return make_row_blocks(hrp, m, cap, rows); },
+            hrp, h->rp, h->ci, E.val, E.XA, E.KXA, n, h->dev_err, &sK, &ms));
+        h->launches += 6 * 4;
+    }
+    if (!E.res.on && !E.slT.on) {
+        LP_TRY(tune_schedule<T>(
+            sms, h->stream, [&](int cap, int rows) { return make_row_blocks(htrp, n, cap, rows); },
+            htrp, h->trp, h->tci, E.tval, E.YA, E.KTYA, m, h->dev_err, &sT, &ms));
+        h->launches += 6 * 4;
+    }
     const bool changed = sK.cap != E.schedK.cap || sK.max_rows != E.schedK.max_rows ||
                          sT.cap != E.schedT.cap || sT.max_rows != E.schedT.max_rows;
     if (changed) {
