@@ -1085,6 +1085,13 @@ void b_launch_attempt(BatchHandle* bh, cudaStream_t st)
         bh->ctrl, bh->meta.B, LK.t0, LT.t0, LK.part, LT.part, LT.n);
 }
 
+// launches of b_launch_check
+template <typename T>
+int b_check_launches(const BatchSched<T>& S)
+{
+    return 8 + (S.slK.on || S.slT.on) + !S.slK.on + !S.slT.on;
+}
+
 template <typename T>
 void b_launch_check(BatchHandle* bh, cudaStream_t st, cudaGraphConditionalHandle hd, int use_handle,
                     int in_body)
@@ -1264,7 +1271,7 @@ lp_status batch_solve_t(BatchHandle* bh, const lp_opts* o, lp_result* rs,
         b_product<T>(bh, true, st, e2, false);
     }
     b_launch_check<T>(bh, st, cudaGraphConditionalHandle{}, 0, 0);
-    h->launches += 11 + 3 + 4;
+    h->launches += b_check_launches(S) + 3 + 4;
     LP_CUDA_TRY(cudaGetLastError());
     auto t_setup = std::chrono::steady_clock::now();
     const int slots = o->check_every + (o->adaptive_step ? 4 : 0);
@@ -1278,7 +1285,7 @@ lp_status batch_solve_t(BatchHandle* bh, const lp_opts* o, lp_result* rs,
     if (derr) return LP_DEVICE_TIMEOUT;
     long long bodies = 0;
     for (const Ctrl& c : hc) bodies = std::max(bodies, c.bodies);
-    h->launches += bodies * (long long)(slots * 4 + 11);
+    h->launches += bodies * (long long)(slots * 4 + b_check_launches(S));
     // solutions, unscaled, stacked; then into each caller's buffers
     double* xo = nullptr;
     LP_TRY(dev_alloc_n(h, &xo, (size_t)(n + m)));

@@ -1,4 +1,5 @@
-"""The schedule autotuner times nothing that a solve does not run."""
+"""The schedule autotuner times nothing that a solve does not run, and the launch counts of
+a sliced batch are those of its launches."""
 import numpy as np
 import pytest
 
@@ -34,3 +35,14 @@ def test_launches_of_the_tuner(L, m, n, row, extra):
         count.append(prob.solve(tol=1e-14, max_iters=8, adaptive_step=0, autotune=tune)[2]["kernel_launches"])
         prob.close()
     assert count[1] - count[0] == extra
+
+
+def test_launches_of_a_sliced_batch(L):
+    """A check period more: 64 attempts of four launches, and a check of nine (one of them
+    lists the slices of the unfinished LPs)."""
+    batch = L.Batch([_lp(13000, 26000, 1), _lp(14000, 28000, 2)])
+    # (the first solve builds the slices)
+    _, a, b = (batch.solve(tol=1e-14, max_iters=k, adaptive_step=0)[0][2]["kernel_launches"]
+               for k in (64, 64, 128))
+    batch.close()
+    assert b - a == 64 * 4 + 9
