@@ -111,15 +111,6 @@ inline long long limit_ns(double s)
     return s >= 9.0e9 ? (long long)9e18 : (long long)(s * 1e9);
 }
 
-// n / d for rd = 1 / d (correctly rounded): the product with rd corrected by its
-// residual, which rounds correctly (Markstein, 1990).  Three fused multiply-adds
-// (200 cycles of GB300's FP64 unit) instead of a division (1,500).
-__host__ __device__ inline double div_by(double n, double d, double rd)
-{
-    const double q = n * rd;
-    return fma(fma(-d, q, n), rd, q);
-}
-
 __host__ __device__ inline void refresh_scalars(Ctrl& c)
 {
     const double tau = div_by(c.eta, c.omega, c.romega), sigma = c.eta * c.omega;

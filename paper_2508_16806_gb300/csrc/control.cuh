@@ -1,7 +1,7 @@
 // Per-LP control decisions of the restarted PDHG loop, shared by the single
-// and the batched solver: the Algorithm 5 step decision and the KKT check
-// (candidate, termination, restart criteria, Algorithm 4).  Each runs in one
-// thread and updates one control block.
+// and the batched solver: the Algorithm 5 step decision, by one thread, and the KKT
+// check (candidate, termination, restart criteria, Algorithm 4), by one warp.  Each
+// updates one control block.
 #pragma once
 
 #include "common.cuh"
@@ -114,74 +114,6 @@ struct ColCheck {
         if (dls < T(0)) v[14] += u * dls;
     }
 };
-
-// The bit pattern of a value as an integer that orders like it (a sign bit turns
-// the order of the rest round; NaNs lie beyond the infinities).
-__device__ __forceinline__ long long order_key(double a)
-{
-    const long long b = __double_as_longlong(a);
-    return b ^ (long long)((unsigned long long)(b >> 63) >> 1);
-}
-
-// v clamped to [lo, hi] (l <= u; a NaN stays).  FP64: on the bit patterns as
-// integers, which order like the values (a sign bit turns the order round): an
-// FP64 comparison would take the FP64 unit.
-__device__ __forceinline__ double res_clamp(double v, double lo, double hi)
-{
-    const long long k = order_key(v);
-    const bool nan = (unsigned long long)(__double_as_longlong(v) & 0x7fffffffffffffffll) >
-                     0x7ff0000000000000ull;
-    double r = v;
-    if (k < order_key(lo)) r = lo;
-    if (k > order_key(hi)) r = hi;
-    return nan ? v : r;
-}
-__device__ __forceinline__ float res_clamp(float v, float lo, float hi)
-{
-    if (v < lo) v = lo;
-    if (v > hi) v = hi;
-    return v;
-}
-// v where it is not negative, else 0 (a NaN stays)
-__device__ __forceinline__ double res_pos(double v)
-{
-    const unsigned long long b = (unsigned long long)__double_as_longlong(v);
-    return b > 0x8000000000000000ull && b <= 0xfff0000000000000ull ? 0.0 : v;
-}
-__device__ __forceinline__ float res_pos(float v) { return v < 0.0f ? 0.0f : v; }
-
-// v > 0, and lo < v < hi (NaNs: false; the zeros are equal), on the bit patterns as well
-__device__ __forceinline__ bool res_positive(double v)
-{
-    const long long b = __double_as_longlong(v);
-    return b > 0 && b <= 0x7ff0000000000000ll;
-}
-__device__ __forceinline__ bool res_positive(float v) { return v > 0.0f; }
-__device__ __forceinline__ bool res_inside(double v, double lo, double hi)
-{
-    long long k = order_key(v), a = order_key(lo), b = order_key(hi);
-    k += k == -1;    // -0
-    a += a == -1;
-    b += b == -1;
-    return a < k && k < b;   // a NaN lies beyond the infinities: no bound is
-}
-__device__ __forceinline__ bool res_inside(float v, float lo, float hi) { return lo < v && v < hi; }
-
-// n / d where both are of ordinary size (and n may be 0): an FP32 reciprocal
-// refined by two Newton steps, the quotient corrected by its residual (Markstein,
-// 1990).  About 600 cycles of the deciding thread, on every attempt's critical
-// path, instead of the 1,500 of a division.
-__device__ __forceinline__ double quotient(double n, double d)
-{
-    const int en = (int)((unsigned long long)__double_as_longlong(n) >> 52) & 2047;
-    const int ed = (int)((unsigned long long)__double_as_longlong(d) >> 52) & 2047;
-    if (ed < 923 || ed > 1123 || (n != 0.0 && (en < 523 || en > 1523))) return n / d;
-    double r = (double)__frcp_rn((float)d);
-    r = fma(r, fma(-d, r, 1.0), r);
-    r = fma(r, fma(-d, r, 1.0), r);
-    const double q = n * r;
-    return fma(fma(-d, q, n), r, q);
-}
 
 // Whether the check kernels evaluate Algorithm 6 for this control block.
 __device__ __forceinline__ bool infeas_active(const Ctrl& c)
