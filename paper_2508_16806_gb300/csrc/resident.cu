@@ -589,11 +589,10 @@ struct SidePlan {
     int chunk = 0, lgmin = 5, max_entry = 0, max_slice = 0, max_slot = 0;
 };
 
-// A row takes one lane up to kResSteps nonzeros (summed in their order), else as many
-// as leave kResSteps each (with more lanes per short row an attempt of the 5,000 x
-// 10,000 LP took 6.0 us instead of 5.4, one of the 200 x 400 LP 4.1 instead of 4.6).
-// cluster: block c owns the rows [c chunk, (c + 1)
-// chunk); otherwise slices of rows sorted within windows of 512 go round the blocks,
+// A row takes one lane up to kResSteps nonzeros, else as many as leave kResSteps each
+// (with more lanes per short row an attempt of the 5,000 x 10,000 LP took 6.0 us instead of
+// 5.4, one of the 200 x 400 LP 4.1 instead of 4.6).  cluster: block c owns the rows
+// [c chunk, (c + 1) chunk); otherwise slices of rows sorted within windows of 512 go round the blocks,
 // those of long rows to the block with the fewest steps.
 SidePlan plan_rows(const std::vector<int64_t>& rp, int nb, bool cluster)
 {

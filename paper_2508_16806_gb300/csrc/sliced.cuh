@@ -6,8 +6,8 @@
 // the nonzeros stored transposed (step k of the 32 lanes side by side, padded to the
 // slice's longest row with column -1).  A warp takes a slice: values and columns
 // come coalesced and without conditions, eight steps in flight, each lane gathers
-// its own row's entries (none for padding) and sums them by fused multiply-adds in
-// order, and the epilogue runs on the row's owner lane.  No shared memory, no row
+// its own row's entries (none for padding) and sums them by fused multiply-adds in a
+// fixed order, and the epilogue runs on the row's owner lane.  No shared memory, no row
 // starts, no hand-over between warps: what is left of the time is the gathers (an SM
 // issues about one 32-byte sector request a cycle) and in FP64 the multiply-adds (16
 // cycles of an SM for a warp's 32 lanes, however few are active: the sorted slices
@@ -54,9 +54,9 @@ __device__ __forceinline__ double gather_if(const double* x, int c)
     return v;
 }
 
-template <int U, typename T>
+template <int U, int C, typename T>
 __device__ __forceinline__ void slice_steps(const int32_t* __restrict__ si, const T* __restrict__ sv,
-                                            const T* x, T& a)
+                                            const T* x, T (&a)[C])
 {
     int c[U];
     T v[U], xv[U];
@@ -67,7 +67,36 @@ __device__ __forceinline__ void slice_steps(const int32_t* __restrict__ si, cons
 #pragma unroll
     for (int u = 0; u < U; ++u) xv[u] = gather_if(x, c[u]);
 #pragma unroll
-    for (int u = 0; u < U; ++u) a = fma(v[u], xv[u], a);
+    for (int u = 0; u < U; ++u) a[u % C] = fma(v[u], xv[u], a[u % C]);
+}
+
+// A lane's n steps in C sums, one for every C-th step, which then meet in pairs: chains as
+// short as those of the ring's lane groups.  Rounding error of an FP64 row sum (root mean
+// square, in 2^-52 of the terms' magnitudes), one chain | 2, 4 from 8 and 8 from 16 steps |
+// the ring: 6 nonzeros 0.20 | 0.19 | 0.20, 12 0.20 | 0.16 | 0.17, 24 0.20 | 0.13 | 0.13, 32 0.20 |
+// 0.12 | 0.12.  The 1M x 2M LP takes 1.8 % longer in FP64, 2.2 % in FP32.
+template <int C, typename T>
+__device__ __forceinline__ T slice_sum(const int32_t* __restrict__ si, const T* __restrict__ sv, int n,
+                                       const T* x)
+{
+    T a[C];
+#pragma unroll
+    for (int k = 0; k < C; ++k) a[k] = T(0);
+    for (; n >= 8; n -= 8, si += 256, sv += 256) slice_steps<8, C, T>(si, sv, x, a);
+    if (n >= 4) {
+        slice_steps<4, C, T>(si, sv, x, a);
+        n -= 4, si += 128, sv += 128;
+    }
+    if (n >= 2) {
+        slice_steps<2, C, T>(si, sv, x, a);
+        n -= 2, si += 64, sv += 64;
+    }
+    if (n >= 1) slice_steps<1, C, T>(si, sv, x, a);
+#pragma unroll
+    for (int o = 1; o < C; o <<= 1)
+#pragma unroll
+        for (int k = 0; k < C; k += 2 * o) a[k] += a[k + o];
+    return a[0];
 }
 
 // One slice: the rows' sums and, on each row's owner lane, their epilogue.
@@ -82,18 +111,10 @@ __device__ __forceinline__ void slice_run(const SlicedSide& S, const T* __restri
     const T* __restrict__ sv = val + (size_t)d.x * 32 + lane;
     typename Epi::Pre pre;
     if (own) pre = epi.load(row);
-    T a = T(0);
-    int n = d.y;
-    for (; n >= 8; n -= 8, si += 256, sv += 256) slice_steps<8, T>(si, sv, x, a);
-    if (n >= 4) {
-        slice_steps<4, T>(si, sv, x, a);
-        n -= 4, si += 128, sv += 128;
-    }
-    if (n >= 2) {
-        slice_steps<2, T>(si, sv, x, a);
-        n -= 2, si += 64, sv += 64;
-    }
-    if (n >= 1) slice_steps<1, T>(si, sv, x, a);
+    T a;
+    if (d.y >= 16) a = slice_sum<8, T>(si, sv, d.y, x);
+    else if (d.y >= 8) a = slice_sum<4, T>(si, sv, d.y, x);
+    else a = slice_sum<2, T>(si, sv, d.y, x);
     for (int o = (1 << d.z) >> 1; o > 0; o >>= 1) a += __shfl_xor_sync(0xffffffffu, a, o);
     if (own) epi.row(row, a, pre, acc);
 }
