@@ -836,7 +836,7 @@ lp_status ensure_sched(BatchHandle* bh)
         const SchedParams d{cap_w<T>(), kTaskRows};
         LP_TRY(build_sched<T>(bh, d, d));
     }
-    if (!S.sliced) {
+    if (!S.sliced && !bh->h.lean) {
         Handle* h = &bh->h;
         LP_TRY(slice_side<T>(h, h->h_rp, h->rp, h->ci, h->n, &bh->meta.row0, &S.slK));
         LP_TRY(slice_side<T>(h, h->h_trp, h->trp, h->tci, h->m, &bh->meta.col0, &S.slT));
@@ -1493,7 +1493,26 @@ static lp_status batch_build(BatchHandle* bh, const lp_handle* hs, int B)
     LP_TRY(dev_alloc_n(h, &bh->lpd, 8 * (size_t)B + 8));
     LP_TRY(dev_alloc_n(h, &bh->go, (size_t)B));
     LP_CUDA_TRY(cudaStreamSynchronize(st));
+    h->base_allocs = h->allocs.size();
     return LP_OK;
+}
+
+// Out of memory: the schedules and engines are given back, and the solve runs once more
+// without slices (as with_room does for one LP).
+lp_status batch_solve(BatchHandle* bh, const lp_opts* o, lp_result* rs)
+{
+    for (;;) {
+        const lp_status s = o->precision == LP_PREC_FP64 ? batch_solve_t<double>(bh, o, rs)
+                                                         : batch_solve_mixed(bh, o, rs);
+        if (s != LP_OUT_OF_MEMORY) return s;
+        release_engines(&bh->h);
+        if (bh->exec) cudaGraphExecDestroy(bh->exec);
+        bh->exec = nullptr;
+        bh->s64 = BatchSched<double>{};
+        bh->s32 = BatchSched<float>{};
+        if (bh->h.lean) return s;
+        bh->h.lean = true;
+    }
 }
 
 }  // namespace pdhg
@@ -1548,10 +1567,8 @@ lp_status lp_batch_solve(lp_batch b, const lp_opts* o, lp_result* rs)
     for (int k = 0; k < b->b.meta.B; ++k)
         if (rs[k].memory_space != LP_MEM_HOST && rs[k].memory_space != LP_MEM_DEVICE)
             return LP_INVALID_ARGUMENT;
-    lp_status s;
-    if (o->precision == LP_PREC_FP64) s = pdhg::batch_solve_t<double>(&b->b, o, rs);
-    else if (o->precision == LP_PREC_MIXED) s = pdhg::batch_solve_mixed(&b->b, o, rs);
-    else return LP_INVALID_ARGUMENT;
+    if (o->precision != LP_PREC_FP64 && o->precision != LP_PREC_MIXED) return LP_INVALID_ARGUMENT;
+    const lp_status s = pdhg::batch_solve(&b->b, o, rs);
     if (s < 0) {
         cudaStreamSynchronize(b->b.h.stream);
         (void)cudaGetLastError();

@@ -32,6 +32,22 @@ void free_all(Handle* h)
     h->stream = nullptr;
 }
 
+// A call that runs out of memory is run once more without what only makes it faster: the
+// second copies of the matrix (resident and sliced forms) and the gradient's packs.  The
+// handle keeps to that, and an engine that is half built is given back.
+template <class F>
+lp_status with_room(Handle* h, F&& call)
+{
+    lp_status s = call();
+    if (s != LP_OUT_OF_MEMORY) return s;
+    release_engines(h);
+    if (h->lean) return s;
+    h->lean = true;
+    s = call();
+    if (s == LP_OUT_OF_MEMORY) release_engines(h);
+    return s;
+}
+
 constexpr double kFp32MaxReflect = 0.5;
 
 lp_status check_opts(const lp_opts* o)
@@ -74,6 +90,25 @@ void fill_result(lp_result* r, const Ctrl& c)
 }
 
 }  // namespace
+
+namespace pdhg {
+
+void release_engines(Handle* h)
+{
+    cudaStreamSynchronize(h->stream);
+    (void)cudaGetLastError();
+    for (auto* E : {&h->e64.exec, &h->e64.body_exec, &h->e32.exec, &h->e32.body_exec})
+        if (*E) cudaGraphExecDestroy(*E);
+    while (h->allocs.size() > h->base_allocs) {
+        cudaFree(h->allocs.back().p);
+        h->allocs.pop_back();
+    }
+    h->e64 = Engine<double>{};
+    h->e32 = Engine<float>{};
+    h->wbuf = nullptr;
+}
+
+}  // namespace pdhg
 
 extern "C" {
 
@@ -358,7 +393,7 @@ static lp_status solve_core(Handle* h, const lp_opts* o, lp_result* r)
 lp_status lp_solve(lp_handle p, const lp_opts* o, lp_result* r)
 {
     if (!p) return LP_INVALID_ARGUMENT;
-    lp_status s = solve_impl(&p->h, o, r);
+    lp_status s = with_room(&p->h, [&] { return solve_impl(&p->h, o, r); });
     if (s < 0) {
         cudaStreamSynchronize(p->h.stream);
         (void)cudaGetLastError();
@@ -394,26 +429,29 @@ lp_status lp_fishnet(lp_handle p, const lp_opts* o, int32_t P, int32_t k_steps, 
     if (check_opts(o) != LP_OK) return LP_INVALID_ARGUMENT;
     if (fishnet_draws(P) > nZ) return LP_INVALID_ARGUMENT;
     Handle* h = &p->h;
-    lp_status s = LP_OK;
-    try {
-        double normK = 0.0, eta0 = 0.0, omega0 = 0.0;
-        s = prepare_fp64(h, o, &normK, &eta0, &omega0);
-        if (s == LP_OK && o->precision == LP_PREC_MIXED) s = setup_engine<float>(h, o);
-        std::vector<double> zh((size_t)nZ);
-        if (s == LP_OK && nZ > 0) {
-            if (memory_space == LP_MEM_HOST) {
-                std::memcpy(zh.data(), Z, sizeof(double) * (size_t)nZ);
-            } else if (cudaMemcpy(zh.data(), Z, sizeof(double) * (size_t)nZ,
-                                  cudaMemcpyDeviceToHost) != cudaSuccess) {
-                s = LP_CUDA_ERROR;
+    lp_status s = with_room(h, [&]() -> lp_status {
+        lp_status s = LP_OK;
+        try {
+            double normK = 0.0, eta0 = 0.0, omega0 = 0.0;
+            s = prepare_fp64(h, o, &normK, &eta0, &omega0);
+            if (s == LP_OK && o->precision == LP_PREC_MIXED) s = setup_engine<float>(h, o);
+            std::vector<double> zh((size_t)nZ);
+            if (s == LP_OK && nZ > 0) {
+                if (memory_space == LP_MEM_HOST) {
+                    std::memcpy(zh.data(), Z, sizeof(double) * (size_t)nZ);
+                } else if (cudaMemcpy(zh.data(), Z, sizeof(double) * (size_t)nZ,
+                                      cudaMemcpyDeviceToHost) != cudaSuccess) {
+                    s = LP_CUDA_ERROR;
+                }
             }
+            if (s == LP_OK)
+                s = run_fishnet(h, o->precision, eta0, omega0, normK, P, k_steps, G, zh.data(), nZ,
+                                x0, y0, gaps, rounds, memory_space);
+        } catch (const std::bad_alloc&) {
+            s = LP_OUT_OF_MEMORY;
         }
-        if (s == LP_OK)
-            s = run_fishnet(h, o->precision, eta0, omega0, normK, P, k_steps, G, zh.data(), nZ,
-                            x0, y0, gaps, rounds, memory_space);
-    } catch (const std::bad_alloc&) {
-        s = LP_OUT_OF_MEMORY;
-    }
+        return s;
+    });
     if (s < 0) {
         cudaStreamSynchronize(h->stream);
         (void)cudaGetLastError();
@@ -429,8 +467,10 @@ lp_status lp_grad(lp_handle p, const lp_opts* o, int32_t K_iters, int32_t ckpt_e
         return LP_INVALID_ARGUMENT;
     if (memory_space != LP_MEM_HOST && memory_space != LP_MEM_DEVICE) return LP_INVALID_ARGUMENT;
     if (check_opts(o) != LP_OK) return LP_INVALID_ARGUMENT;
-    lp_status s = run_grad(&p->h, o, K_iters, ckpt_every, dL_dxK, dc, dq, dvals, x_K,
-                           memory_space, tau_sigma_out);
+    lp_status s = with_room(&p->h, [&] {
+        return run_grad(&p->h, o, K_iters, ckpt_every, dL_dxK, dc, dq, dvals, x_K, memory_space,
+                        tau_sigma_out);
+    });
     if (s < 0) {
         cudaStreamSynchronize(p->h.stream);
         (void)cudaGetLastError();
@@ -445,7 +485,9 @@ lp_status lp_unroll(lp_handle p, const lp_opts* o, int32_t K_iters, double* x_K,
     if (memory_space != LP_MEM_HOST && memory_space != LP_MEM_DEVICE) return LP_INVALID_ARGUMENT;
     lp_status s = check_opts(o);
     if (s != LP_OK) return s;
-    s = run_unroll(&p->h, o, K_iters, x_K, y_K, memory_space, tau_sigma_out);
+    s = with_room(&p->h, [&] {
+        return run_unroll(&p->h, o, K_iters, x_K, y_K, memory_space, tau_sigma_out);
+    });
     if (s < 0) {
         cudaStreamSynchronize(p->h.stream);
         (void)cudaGetLastError();

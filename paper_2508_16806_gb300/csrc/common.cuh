@@ -307,6 +307,8 @@ struct Handle {
     double* wbuf = nullptr;      // [n + m] scaled FP64 hand-off state (mixed precision polish)
     int* dev_err = nullptr;      // device flag: a bounded wait of a kernel gave up
     std::vector<DevBuf> allocs;
+    size_t base_allocs = 0;      // those of the problem itself; the rest can be built again
+    bool lean = false;           // a call ran out of memory: no second copy of the matrix
     Engine<double> e64;
     Engine<float> e32;
     long long launches = 0;      // kernels launched by the host (graph bodies counted apart)
@@ -605,6 +607,8 @@ template <typename T>
 lp_status profile_step(Handle* h, int reps, double* ms, double* bytes);
 // resident.cu: the plan of an engine (res.on false: the LP is too large), the
 // attempts of one check period, Algorithm 2 from ones (||K b / ||b|| ||^2 -> out)
+// capi.cu: gives back what the engines hold (they are built again by the next call)
+void release_engines(Handle* h);
 template <typename T> lp_status res_plan(Handle* h);
 template <typename T> lp_status res_values(Handle* h);   // the slices' values from val, tval
 template <typename T> lp_status launch_res_period(Handle* h, cudaStream_t st, bool halpern);

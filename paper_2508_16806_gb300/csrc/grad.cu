@@ -398,7 +398,7 @@ lp_status grad_impl(Handle* h, const lp_opts* o, int K, int ckpt, const double* 
     // reverse pass
     T *RX = nullptr, *RY = nullptr, *gx = nullptr, *gy = nullptr, *gvx = nullptr, *gvy = nullptr;
     double2 *P = nullptr, *Q = nullptr;
-    const int S = std::min(kGSteps, ckpt);   // reverse steps packed together
+    const int S = h->lean ? 1 : std::min(kGSteps, ckpt);   // reverse steps packed together
     uint8_t *RMX = nullptr, *RMY = nullptr;
     double *ddc = nullptr, *ddq = nullptr, *ddv = nullptr;
     LP_TRY(B.alloc((void**)&RX, sizeof(T) * (size_t)(ckpt + 1) * n));

@@ -842,6 +842,7 @@ lp_status setup_create(Handle* h, const lp_desc* d)
     h->qnorm = std::sqrt(s);
     LP_TRY(sum_of_squares(h, h->c0, n, &s));
     h->cnorm = std::sqrt(s);
+    h->base_allocs = h->allocs.size();
     return LP_OK;
 }
 
@@ -1155,8 +1156,8 @@ lp_status setup_engine(Handle* h, const lp_opts* o)
     const int64_t m = h->m, n = h->n, nnz = h->nnz;
     Engine<T>& E = engine_of<T>(h);
     if (!E.ready) {
-        LP_TRY(res_plan<T>(h));
-        if (!E.res.on) LP_TRY(slice_plan<T>(h));
+        if (!h->lean) LP_TRY(res_plan<T>(h));
+        if (!h->lean && !E.res.on) LP_TRY(slice_plan<T>(h));
         // the K side gathers x (n entries), the K^T side y (m entries)
         LP_TRY(engine_schedule<T>(h, SchedParams{spmv_cap<T>(n), kTaskRows},
                                   SchedParams{spmv_cap<T>(m), kTaskRows}));

@@ -152,16 +152,18 @@ lp_status slice_side(Handle* h, const std::vector<int64_t>& hrp, const int64_t* 
         steps += c.y;
         nl += c.z;
     }
-    // a second copy of the matrix: only where memory is plentiful
+    // A second copy of the matrix: at most a sixteenth of the device's memory, so a quarter
+    // for both sides in both precisions.  (By what is free, the same LP summed in another
+    // order when something else held the card.)
     size_t avail = 0, total = 0;
     LP_CUDA_TRY(cudaMemGetInfo(&avail, &total));
     const size_t need = (size_t)ns * sizeof(int4) + (size_t)nl * 4 + (size_t)steps * 32 * (8 + sizeof(T));
-    if (steps * 32 >= ((int64_t)1 << 31) || nl >= ((int64_t)1 << 31) || need > avail / 4) {
-        return LP_OK;
-    }
-    // one allocation: values, records, columns, nonzeros, rows
+    if (steps * 32 >= ((int64_t)1 << 31) || nl >= ((int64_t)1 << 31) || need > total / 16) return LP_OK;
+    // one allocation: values, records, columns, nonzeros, rows; without room the ring stays
     T* val = nullptr;
-    LP_TRY(dev_alloc(h, (void**)&val, need));
+    const lp_status as = dev_alloc(h, (void**)&val, need);
+    if (as == LP_OUT_OF_MEMORY) return LP_OK;
+    LP_TRY(as);
     int4* raw = reinterpret_cast<int4*>(val + steps * 32);
     int32_t* idx = reinterpret_cast<int32_t*>(raw + ns);
     int32_t* perm = idx + steps * 32;
