@@ -974,19 +974,22 @@ static lp_status build_graph(Handle* h, Engine<T>& E, int check_every, int slots
     if (conditional) {
         LP_CUDA_TRY(cudaStreamBeginCaptureToGraph(st, body, nullptr, nullptr, 0,
                                                   cudaStreamCaptureModeThreadLocal));
-        LP_TRY(launch_attempts<T>(h, E, st, slots, halpern != 0));
+        // (a launch that fails does not leave the caller's stream capturing)
+        const lp_status ls = launch_attempts<T>(h, E, st, slots, halpern != 0);
         launch_check<T>(h, E, st, hd, 1, 1, halpern != 0);
         cudaGraph_t captured = nullptr;
         LP_CUDA_TRY(cudaStreamEndCapture(st, &captured));
+        LP_TRY(ls);
         LP_CUDA_TRY(cudaGraphInstantiate(&E.exec, graph, 0));
         cudaGraphDestroy(graph);
     } else {
         cudaGraphDestroy(graph);
         LP_CUDA_TRY(cudaStreamBeginCapture(st, cudaStreamCaptureModeThreadLocal));
-        LP_TRY(launch_attempts<T>(h, E, st, slots, halpern != 0));
+        const lp_status ls = launch_attempts<T>(h, E, st, slots, halpern != 0);
         launch_check<T>(h, E, st, hd, 0, 1, halpern != 0);
         cudaGraph_t g2 = nullptr;
         LP_CUDA_TRY(cudaStreamEndCapture(st, &g2));
+        LP_TRY(ls);
         LP_CUDA_TRY(cudaGraphInstantiate(&E.body_exec, g2, 0));
         cudaGraphDestroy(g2);
     }
