@@ -6,6 +6,8 @@
 #include <type_traits>
 #include <vector>
 
+#include <cuda.h>
+
 #include "resident.cuh"
 
 namespace pdhg {
@@ -737,6 +739,30 @@ lp_status res_launch(const ResPlan& R, cudaStream_t st, const void* f, void** ar
 
 constexpr size_t kResSmem = 227 * 1024 - 4096;   // of a block, less the kernels' static part
 
+// SMs that the kernels of a stream may use: those of its green context, or of its context
+// (the device's where the driver does not say).
+int stream_sms(cudaStream_t st, int device_sms)
+{
+    const auto entry = [](const char* name, unsigned version) {
+        void* f = nullptr;
+        cudaDriverEntryPointQueryResult r = cudaDriverEntryPointSymbolNotFound;
+        if (cudaGetDriverEntryPointByVersion(name, &f, version, cudaEnableDefault, &r) != cudaSuccess)
+            (void)cudaGetLastError();
+        return r == cudaDriverEntryPointSuccess ? f : nullptr;
+    };
+    const auto get = reinterpret_cast<decltype(&cuStreamGetCtx_v2)>(entry("cuStreamGetCtx", 12050));
+    const auto of_green =
+        reinterpret_cast<decltype(&cuGreenCtxGetDevResource)>(entry("cuGreenCtxGetDevResource", 12040));
+    const auto of_ctx = reinterpret_cast<decltype(&cuCtxGetDevResource)>(entry("cuCtxGetDevResource", 12040));
+    CUcontext ctx = nullptr;
+    CUgreenCtx green = nullptr;
+    CUdevResource res;
+    if (!get || !of_green || !of_ctx || get(st, &ctx, &green) != CUDA_SUCCESS) return device_sms;
+    const CUresult r = green ? of_green(green, &res, CU_DEV_RESOURCE_TYPE_SM)
+                             : of_ctx(ctx, &res, CU_DEV_RESOURCE_TYPE_SM);
+    return r == CUDA_SUCCESS ? (int)res.sm.smCount : device_sms;
+}
+
 }  // namespace
 
 template <typename T>
@@ -750,6 +776,9 @@ lp_status res_plan(Handle* h)
     int sms = 0, coop = 0;
     LP_CUDA_TRY(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, h->device));
     LP_CUDA_TRY(cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, h->device));
+    // the blocks of a launch wait for one another: on a part of the device, which may not
+    // hold them all at once, the launches per product stay
+    if (stream_sms(h->stream, sms) < sms) return LP_OK;
     sms = std::min(sms, kResMaxGrid);
     // Resident only where nonzeros and state fit the chip's shared memory (34 MB: about
     // 1.2M nonzeros in FP32 at 12 a row): with the nonzeros left in L2 an attempt of the
