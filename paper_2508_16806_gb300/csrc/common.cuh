@@ -420,7 +420,7 @@ __device__ __forceinline__ double warp_max_nonneg(double v)
         const unsigned long long u = __shfl_xor_sync(0xffffffffu, b, o);
         b = u > b ? u : b;
     }
-    return __longlong_as_double((long long)b);
+    return bits_double((long long)b);
 }
 
 // Block sums of NS <= 16 and maxima of NM non-negative values per thread:
@@ -460,51 +460,6 @@ __device__ __forceinline__ double warp_max(double v)
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) v = fmax(v, __shfl_down_sync(0xffffffffu, v, o));
     return v;
-}
-
-// Block maxima of NQ per-thread values into part[q * stride + blockIdx.x].
-template <int NQ, int NT>
-__device__ __forceinline__ void block_partials_max(const double (&v)[NQ], double* part, int stride)
-{
-    __shared__ double sh[NQ][NT / 32];
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-#pragma unroll
-    for (int q = 0; q < NQ; ++q) {
-        double t = warp_max(v[q]);
-        if (lane == 0) sh[q][warp] = t;
-    }
-    __syncthreads();
-    if (warp == 0) {
-#pragma unroll
-        for (int q = 0; q < NQ; ++q) {
-            double t = lane < NT / 32 ? sh[q][lane] : -INFINITY;
-            t = warp_max(t);
-            if (lane == 0) part[(size_t)q * stride + blockIdx.x] = t;
-        }
-    }
-}
-
-// Maximum of part[0..count) by a whole block (valid in every thread).
-template <int NT>
-__device__ double block_max_array(const double* part, int count)
-{
-    __shared__ double sh[NT / 32];
-    __shared__ double total;
-    double s = -INFINITY;
-    for (int i = threadIdx.x; i < count; i += NT) s = fmax(s, __ldcg(part + i));
-    s = warp_max(s);
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    if (lane == 0) sh[warp] = s;
-    __syncthreads();
-    if (warp == 0) {
-        double t = lane < NT / 32 ? sh[lane] : -INFINITY;
-        t = warp_max(t);
-        if (lane == 0) total = t;
-    }
-    __syncthreads();
-    double r = total;
-    __syncthreads();
-    return r;
 }
 
 // Fixed-order sum of part[0..count) by a whole block of NT threads; the
