@@ -201,18 +201,19 @@ __device__ __forceinline__ void step_decide(Ctrl* ctrl, int adapt, double dy2, d
     }
     // guards that end the device loop even if no check is reached: Algorithm 5
     // accepts once eta <= 1/||K||, so a long run of rejections means broken
-    // arithmetic; the wall-clock limit is also enforced per attempt.
+    // arithmetic; the wall-clock limit is also enforced per attempt (by the check
+    // itself where one follows: a Halpern iteration has then written the candidate,
+    // which without that check would not be the one of the last record).
     if (ctrl->rejects > 1000 || order_key(eta_next) <= 0 ||
         order_key(eta_next) > 0x7ff0000000000000ll) {
         ctrl->status = LP_NUMERICAL_ERROR;
         ctrl->done = 1;
         ctrl->skip = 1;
         ctrl->want_check = 0;
-    } else if ((long long)now - ctrl->t0_ns > ctrl->time_limit_ns) {
+    } else if (!ctrl->want_check && (long long)now - ctrl->t0_ns > ctrl->time_limit_ns) {
         ctrl->status = LP_TIME_LIMIT;
         ctrl->done = 1;
         ctrl->skip = 1;
-        ctrl->want_check = 0;
     }
 }
 
