@@ -327,7 +327,9 @@ lp_status lp_update_values(lp_handle h, const double* vals, const double* c, con
  * receives the mean milliseconds per launch of: [0] primal update,
  * [1] K x' SpMV + dual update, [2] K^T y' SpMV + step terms, [3] step control.
  * bytes_out (host, 4 doubles, or NULL) receives the algorithmic bytes per launch
- * of the same kernels.  The solver state afterwards is unspecified. */
+ * of the same kernels.  (An LP small enough to be solved by resident launches is
+ * timed by the launches per product that it does not take in lp_solve.)  The solver
+ * state afterwards is unspecified. */
 lp_status lp_profile_step(lp_handle h, int32_t precision, int32_t reps, double* ms_out,
                           double* bytes_out);
 

@@ -54,7 +54,7 @@ __device__ __forceinline__ double gather_if(const double* x, int c)
     return v;
 }
 
-template <int U, int C, typename T>
+template <int U, int M, int C, typename T>
 __device__ __forceinline__ void slice_steps(const int32_t* __restrict__ si, const T* __restrict__ sv,
                                             const T* x, T (&a)[C])
 {
@@ -67,14 +67,17 @@ __device__ __forceinline__ void slice_steps(const int32_t* __restrict__ si, cons
 #pragma unroll
     for (int u = 0; u < U; ++u) xv[u] = gather_if(x, c[u]);
 #pragma unroll
-    for (int u = 0; u < U; ++u) a[u % C] = fma(v[u], xv[u], a[u % C]);
+    for (int u = 0; u < U; ++u) a[u % M] = fma(v[u], xv[u], a[u % M]);
 }
 
-// A lane's n steps in C sums, one for every C-th step, which then meet in pairs: chains as
-// short as those of the ring's lane groups.  Rounding error of an FP64 row sum (root mean
-// square, in 2^-52 of the terms' magnitudes), one chain | 2, 4 from 8 and 8 from 16 steps |
-// the ring: 6 nonzeros 0.20 | 0.19 | 0.20, 12 0.20 | 0.16 | 0.17, 24 0.20 | 0.13 | 0.13, 32 0.20 |
-// 0.12 | 0.12.  The 1M x 2M LP takes 1.8 % longer in FP64, 2.2 % in FP32.
+// A lane's n steps in C sums, one for every C-th step of the groups of eight (what is left
+// in two of them), which then meet in pairs: chains as short as those of the ring's lane
+// groups.  Rounding error of an FP64 row sum (root mean square, in 2^-52 of the terms'
+// magnitudes), one chain | four sums, eight from 16 steps | the ring: 6 nonzeros 0.20 | 0.19 |
+// 0.20, 12 0.20 | 0.17 | 0.17, 24 0.20 | 0.13 | 0.13, 32 0.20 | 0.12 | 0.12; FP32 with four: 12
+// 0.17 | 0.19 (ring), 24 0.14 | 0.15, 32 0.13 | 0.13.  The 1M x 2M LP, K and K^T side, one chain ->
+// so: FP64 146 + 110 -> 154 + 112 us, FP32 111 + 99 -> 113 + 98 (116 with sums for two, four and
+// eight chosen by a branch).
 template <int C, typename T>
 __device__ __forceinline__ T slice_sum(const int32_t* __restrict__ si, const T* __restrict__ sv, int n,
                                        const T* x)
@@ -82,16 +85,16 @@ __device__ __forceinline__ T slice_sum(const int32_t* __restrict__ si, const T* 
     T a[C];
 #pragma unroll
     for (int k = 0; k < C; ++k) a[k] = T(0);
-    for (; n >= 8; n -= 8, si += 256, sv += 256) slice_steps<8, C, T>(si, sv, x, a);
+    for (; n >= 8; n -= 8, si += 256, sv += 256) slice_steps<8, C, C, T>(si, sv, x, a);
     if (n >= 4) {
-        slice_steps<4, C, T>(si, sv, x, a);
+        slice_steps<4, 2, C, T>(si, sv, x, a);
         n -= 4, si += 128, sv += 128;
     }
     if (n >= 2) {
-        slice_steps<2, C, T>(si, sv, x, a);
+        slice_steps<2, 2, C, T>(si, sv, x, a);
         n -= 2, si += 64, sv += 64;
     }
-    if (n >= 1) slice_steps<1, C, T>(si, sv, x, a);
+    if (n >= 1) slice_steps<1, 2, C, T>(si, sv, x, a);
 #pragma unroll
     for (int o = 1; o < C; o <<= 1)
 #pragma unroll
@@ -112,9 +115,8 @@ __device__ __forceinline__ void slice_run(const SlicedSide& S, const T* __restri
     typename Epi::Pre pre;
     if (own) pre = epi.load(row);
     T a;
-    if (d.y >= 16) a = slice_sum<8, T>(si, sv, d.y, x);
-    else if (d.y >= 8) a = slice_sum<4, T>(si, sv, d.y, x);
-    else a = slice_sum<2, T>(si, sv, d.y, x);
+    if (sizeof(T) == 8 && d.y >= 16) a = slice_sum<8, T>(si, sv, d.y, x);
+    else a = slice_sum<4, T>(si, sv, d.y, x);
     for (int o = (1 << d.z) >> 1; o > 0; o >>= 1) a += __shfl_xor_sync(0xffffffffu, a, o);
     if (own) epi.row(row, a, pre, acc);
 }
