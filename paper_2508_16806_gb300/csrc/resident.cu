@@ -784,7 +784,7 @@ lp_status res_plan(Handle* h)
     // 1.2M nonzeros in FP32 at 12 a row): with the nonzeros left in L2 an attempt of the
     // 100,000 x 200,000 LP (1.25M nonzeros, FP32, Halpern) took 27 us, as the launches
     // per product do.  Within it the grid form is the better one up to its largest size
-    // (50,000 x 100,000 in FP64: 17.5 us an attempt against 38), the cluster form
+    // (50,000 x 100,000 in FP64: 16.4 us an attempt against 37.6), the cluster form
     // wherever it fits (5,000 x 10,000 in FP32: 5.0 us against 10.8 for the grid).
     const double need = 2.0 * (double)nnz * (sizeof(T) + 4) + (double)m * (4 + kResRowT * sizeof(T) + 1) +
                         (double)n * (4 + kResColT * sizeof(T) + 1);

@@ -18,9 +18,10 @@
 // the gathered vectors; a block sends its new entries to the others by bulk
 // copies that complete on the receivers' mbarriers, which is the barrier.
 // Otherwise a cooperative grid gathers through L2 and meets at a barrier in
-// global memory.  An attempt takes (launches per product -> resident): 200 x 400,
-// FP64 19.8 -> 4.5 us; 5,000 x 10,000, FP32 17.5 -> 5.0 us; 20,000 x 40,000, FP64
-// with adaptive steps 35 -> 14 us; 50,000 x 100,000, FP64 40.8 -> 17.5 us.  The
+// global memory.  An attempt takes (launches per product -> resident,
+// a check per 1,024): 200 x 400, FP64 19.2 -> 3.9 us; 5,000 x 10,000, FP32 15.1 -> 4.2 us,
+// FP64 20.5 -> 8.0 us; 20,000 x 40,000, FP64 with adaptive steps 31.5 -> 12.6 us; 50,000 x
+// 100,000, FP64 37.6 -> 16.4 us; 100,000 x 200,000, FP32 26.6 -> 22.1 us.  The
 // cluster form is bound by its barriers (two of about 1,200 cycles an attempt) and
 // the latency of a slice; the grid form by its gathers (a 32-byte sector each, one
 // a cycle and SM) and barriers (2,500 cycles each).
